@@ -99,6 +99,7 @@ struct Ctrl {
     int n_found;           // colliding pairs found
     int n_resolved;        // colliding pairs resolved (collision resolution on)
     int walk_iters;
+    int resort_bad;        // the key sort in progress found its kept keys out of order
     int resort_ok;         // the last key sort took the nearly-sorted path (1) or the radix sort
     int n_m2l_dir;
     int n_p2p_dir;

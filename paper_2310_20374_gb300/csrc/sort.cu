@@ -698,7 +698,7 @@ __global__ void __launch_bounds__(RZ_T) k_resort(ResortArgs A) {
     const int n = A.n, G = gridDim.x, b = blockIdx.x, t = threadIdx.x;
     const int chunk = (n + G - 1) / G, c0 = min(n, b * chunk), c1 = min(n, c0 + chunk);
     unsigned bar = 0;
-    if (b == 0 && t == 0) A.ctl->resort_ok = 0;
+    if (b == 0 && t == 0) A.ctl->resort_ok = A.ctl->resort_bad = 0;
     // ---- 1. movers per block
     int mine = 0;
     for (int i = c0 + t; i < c1; i += RZ_T) mine += is_mover(A.key, i, n) ? 1 : 0;
@@ -746,7 +746,7 @@ __global__ void __launch_bounds__(RZ_T) k_resort(ResortArgs A) {
     {
         bool bad = false;
         for (int p = b * RZ_T + t; p + 1 < ns; p += G * RZ_T) bad |= __ldcg(&A.s_key[p]) > __ldcg(&A.s_key[p + 1]);
-        if (__syncthreads_or(bad) && t == 0) A.ctl->resort_ok = -1;
+        if (__syncthreads_or(bad) && t == 0) A.ctl->resort_ok = A.ctl->resort_bad = -1;
     }
     const bool by_rank = nm <= RS_MOVERS_SMEM;   // uniform
     if (by_rank) {
@@ -776,7 +776,9 @@ __global__ void __launch_bounds__(RZ_T) k_resort(ResortArgs A) {
         if (!radix_body(R, bar)) return;
     }
     if (!grid_sync(A.ctl, bar)) return;
-    if (*reinterpret_cast<volatile int *>(&A.ctl->resort_ok) != 0) {   // stayers out of order (uniform)
+    // stayers out of order: the same for every thread of every block (resort_ok is not, block 0 sets it at
+    // its end, which a late block must not take for this)
+    if (*reinterpret_cast<volatile int *>(&A.ctl->resort_bad) != 0) {
         radix_body(A.radix, bar);
         return;
     }
