@@ -103,6 +103,7 @@ struct Ctrl {
     int resort_ok;         // the last key sort took the nearly-sorted path (1) or the radix sort
     int n_m2l_dir;
     int n_p2p_dir;
+    int n_near;            // near-field work items
     unsigned bar_count;
     unsigned bar_count2;   // grid barriers of the collision climb (it may run beside another cooperative kernel
                            // of the same tree set)

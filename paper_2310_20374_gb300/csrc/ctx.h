@@ -65,6 +65,8 @@ struct WalkLists {
     int2 *m2l_dir = nullptr;      // (target, source) grouped by target
     int *p2p_off = nullptr;       // [cap+1] offsets of each target leaf's sources
     int2 *p2p_src = nullptr;      // each directed entry's source leaf as (first moonlet, moonlet count)
+    int4 *near_items = nullptr;   // near-field work items: (first moonlet, +-count, entries [s0, s1) of p2p_src)
+    int near_cap = 0;
     int2 *cp2p = nullptr;         // collision walk: leaf pairs to test [p2p_cap]
     int *cself = nullptr;         // collision walk: leaves to test within [self_cap]
 };
@@ -81,6 +83,26 @@ struct TreeSet {
 };
 
 constexpr int WALK_MAX_ITERS = 96;
+
+// Near-field work items (near.cu): some of a leaf's moonlets and a share of its
+// direct entries.  The mixed kernel takes an item's m targets two per lane in
+// G = floor(32 / ceil(m / 2)) groups, so 33 to 52 targets (one group, 52 to 81 %
+// of the lanes) go better as 32 (two groups, every lane) and the rest, although
+// the sources are then staged twice.
+__host__ __device__ inline int near_targets(int m) { return m > 64 ? 64 : (m > 32 && m <= 52 ? 32 : m); }
+
+// Equal shares of E direct entries for m targets: NEAR_ENTRIES G source leaves
+// of some sixteen moonlets each are about forty rounds of the kernel's loop
+// whatever m is; with few leaves the shares shrink until there are several
+// items per warp of the device, down to four entries (an item's fixed cost is
+// about that of four).
+constexpr int NEAR_ENTRIES = 10, NEAR_ENTRIES_MIN = 4, NEAR_ITEMS_WANTED = 8192;
+__host__ __device__ inline int near_shares(int E, int m, int n_leaves) {
+    long long e = NEAR_ENTRIES * (32 / ((m + 1) / 2));
+    if (n_leaves < NEAR_ITEMS_WANTED) e = e * n_leaves / NEAR_ITEMS_WANTED;
+    const int per = e < NEAR_ENTRIES_MIN ? NEAR_ENTRIES_MIN : static_cast<int>(e);
+    return (E + per - 1) / per;
+}
 
 // Grid of a cooperative launch: the given blocks per SM, capped by the
 // context's limit so that the cooperative grids of contexts driven on
@@ -253,13 +275,15 @@ struct ExtForce {
     double inv_rs2;        // 1 / r_star^2
     double bulge;          // G M_c R_c^2 J2 of the equatorial bulge (0: off)
 };
-void launch_near(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G);
 // Algorithm StandardTree for the moonlets of S (tree order) on the current tree, whose geometry and
 // multipoles are computed: S.ax = mutual + external, amx = mutual (want_mutual)
 void launch_standard(ncorp_ctx *c, const ParticleSet &S, int n, int p, bool mixed, double G, ExtForce ext,
                      bool want_mutual, int pre, int post);
 void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G, ExtForce ext, bool want_mutual,
                 double kick_h = 0.0);
+
+// ---- near.cu ----
+void launch_near(ncorp_ctx *c, const ParticleSet &P, bool mixed, double G);
 
 // ---- collide.cu ----
 // the box of (x, y, z) emptied and folded again into ctl when *gate != 0 (decided on the device)

@@ -1,21 +1,12 @@
 // eval.cu -- tree descent and evaluation at the moonlets: the complete local
 // expansion of every cell (Sect. 3.4.3, Eq. shifting), L2P at the moonlets,
-// the direct ("brute force") gravity of each leaf's near-field list, and the
-// central-body / distant-star forces (App. B.1, B.3).
+// and the central-body / distant-star forces (App. B.1, B.3).
 //
-// Evaluation in two kernels, so that the near field (which needs only the
-// direct lists) can run while M2L and the descent produce the local
-// expansions.  k_eval: every moonlet gets
-//   sum_j mu_j (x_j - x)/|x_j - x|^3 over the moonlets of its leaf's direct list
-// (mu_j = G m_j; coincident pairs, the moonlet itself included, are skipped).
-// k_far: it adds
+// Evaluation in two kernels, so that the near field (near.cu, which needs only
+// the direct lists) can run while M2L and the descent produce the local
+// expansions.  k_far adds to a moonlet's near-field sum
 //   a = (1/rho) sum_{|beta| <= p-1} C-hat_{e_k+beta} (d/rho)^beta / beta!,  d = x - s_leaf,
 // from its leaf's complete local expansion, and the external forces in FP64.
-//
-// Mixed precision: the direct sum reads every position as an FP32 pair
-// (hi, lo) with x = hi + lo; (hi_j - hi_i) + (lo_j - lo_i) gives the
-// separation to ~1e-7 relative at any distance, so no FP64 work is done per
-// pair.
 #include <type_traits>
 
 #include "ctx.h"
@@ -47,9 +38,6 @@ struct EvalArgs {
     const float4 *gh, *gl;
     const void *Cf;   // complete local expansions
     const float *Cf_lo;   // mixed: low parts of their order-1 coefficients
-    const int *p2p_off;
-    const int2 *p2p_src;      // per directed entry: the source leaf's (first, count)
-    int p2p_dir_cap;
     const double *x, *y, *z, *m;
     const float4 *hi4, *lo4;
     double G;
@@ -59,7 +47,6 @@ struct EvalArgs {
     double *nx, *ny, *nz;     // near-field sums per moonlet (tree order)
     double kick_h;            // k_far: v += kick_h a after the evaluation (0: no kick)
     double *vx, *vy, *vz;
-    int *work;
     const Ctrl *ctl;
 };
 
@@ -318,177 +305,6 @@ __global__ void __launch_bounds__(32 * DESC_WARPS) k_descend(DescendArgs A) {
     }
 }
 
-// ---------------------------------------------------------------------------
-// Evaluation kernel: one block of EV_THREADS threads per leaf, leaves handed
-// out dynamically.  The leaf's m targets (taken EV_THREADS at a time if the
-// leaf is larger) are taken by G = floor(EV_THREADS / m) groups of m threads:
-// thread (g, t) sums the staged sources k = g, g + G, g + 2G, ... for target
-// t, so a leaf of a few moonlets keeps the lanes busy.  The direct list is
-// staged EV_BUF moonlets at a time, cutting source leaves where the buffer
-// ends.  Mixed precision: every thread adds its FP32 partial sum to a
-// double-float total every 32 sources (two-sum), and the groups' totals are
-// added in group order, so that the rounding of a long FP32 running sum
-// (dominated by the nearest pull) does not grow with the direct list.
-// ---------------------------------------------------------------------------
-constexpr int EV_THREADS = 128;
-constexpr int EV_BUF = 512;
-
-template <int P, typename real>
-struct EvShared {
-    __align__(16) unsigned char buf[EV_BUF * 32];   // FP32: float4 hi[EV_BUF] (xyz, mu), lo[EV_BUF]
-                                                    // FP64: double x, y, z, mu [EV_BUF]
-    real red[6][EV_THREADS];
-    int lfirst[32], lpre[32];
-    int leaf, total, next_si, next_soff;
-};
-
-template <int P, typename real>
-__global__ void __launch_bounds__(EV_THREADS, 6) k_eval(EvalArgs A) {
-    constexpr bool f32 = std::is_same<real, float>::value;
-    __shared__ EvShared<P, real> S;
-    if (aborted(A.ctl)) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int nl = A.ctl->n_leaves;
-    float4 *sh = reinterpret_cast<float4 *>(S.buf), *sl = sh + EV_BUF;
-    double *bx = reinterpret_cast<double *>(S.buf), *by = bx + EV_BUF, *bz = by + EV_BUF, *bm = bz + EV_BUF;
-    while (true) {
-        __syncthreads();
-        if (tid == 0) S.leaf = atomicAdd(A.work, 1);
-        __syncthreads();
-        const int li = S.leaf;
-        if (li >= nl) break;
-        const int leaf = A.leaves[li];
-        const int f = A.first[leaf], cnt = A.count[leaf];
-        const int s0 = min(A.p2p_off[leaf], A.p2p_dir_cap), s1 = min(A.p2p_off[leaf + 1], A.p2p_dir_cap);
-        for (int t0 = 0; t0 < cnt; t0 += EV_THREADS) {
-            const int m = min(EV_THREADS, cnt - t0);
-            const int G = EV_THREADS / m, g = tid / m, tt = tid - g * m;
-            const bool act = g < G;   // the last EV_THREADS - G m threads only help with staging
-            const int i = f + t0 + (act ? tt : 0);
-            const float4 th = A.hi4[i], tl = A.lo4[i];
-            const double X = A.x[i], Y = A.y[i], Z = A.z[i];
-            real ax = real(0), ay = real(0), az = real(0);
-            // mixed: double-float totals, to which the FP32 partial sums are added every 32 sources
-            float h3[3] = {0.f, 0.f, 0.f}, l3[3] = {0.f, 0.f, 0.f};
-            int si = s0, soff = 0;
-            while (si < s1) {
-                __syncthreads();
-                if (warp == 0) {
-                    const int idx = si + lane;
-                    int fst = 0, c = 0;
-                    if (idx < s1) {
-                        const int2 e = A.p2p_src[idx];
-                        fst = e.x;
-                        c = e.y;
-                    }
-                    if (lane == 0) { fst += soff; c -= soff; }
-                    int inc = c;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const int v = __shfl_up_sync(0xffffffffu, inc, o);
-                        if (lane >= o) inc += v;
-                    }
-                    const int exc = inc - c;
-                    const int total = min(EV_BUF, __shfl_sync(0xffffffffu, inc, 31));
-                    S.lfirst[lane] = fst;
-                    S.lpre[lane] = exc;
-                    // source leaves consumed completely; the next one may be cut
-                    const unsigned done = __ballot_sync(0xffffffffu, idx < s1 && inc <= total);
-                    const int L = __popc(done);
-                    const int excL = __shfl_sync(0xffffffffu, exc, L & 31);
-                    if (lane == 0) {
-                        S.total = total;
-                        S.next_si = si + L;
-                        S.next_soff = (L < 32 && si + L < s1) ? (L == 0 ? soff : 0) + (total - excL) : 0;
-                    }
-                }
-                __syncthreads();
-                const int total = S.total;
-                for (int t = tid; t < total; t += EV_THREADS) {
-                    int q = 0;
-#pragma unroll
-                    for (int st = 16; st > 0; st >>= 1)
-                        if (S.lpre[q + st] <= t) q += st;
-                    const int jj = S.lfirst[q] + t - S.lpre[q];
-                    if constexpr (f32) {
-                        sh[t] = A.hi4[jj];
-                        sl[t] = A.lo4[jj];
-                    } else {
-                        bx[t] = A.x[jj];
-                        by[t] = A.y[jj];
-                        bz[t] = A.z[jj];
-                        bm[t] = A.G * A.m[jj];
-                    }
-                }
-                si = S.next_si;
-                soff = S.next_soff;
-                __syncthreads();
-                if (act) {
-                    if constexpr (f32) {
-                        for (int k0 = g; k0 < total; k0 += 32 * G) {
-                            const int k1 = min(total, k0 + 32 * G);
-#pragma unroll 4
-                            for (int k = k0; k < k1; k += G) p2p_f32(sh[k], sl[k], th, tl, ax, ay, az);
-                            df_add(h3[0], l3[0], ax); df_add(h3[1], l3[1], ay); df_add(h3[2], l3[2], az);
-                            ax = ay = az = 0.f;
-                        }
-                    } else {
-#pragma unroll 2
-                        for (int k = g; k < total; k += G) p2p_f64(bx[k], by[k], bz[k], bm[k], X, Y, Z, ax, ay, az);
-                    }
-                }
-            }
-            if constexpr (f32) {   // the groups' double-float totals, added in group order
-                if (G > 1) {
-                    __syncthreads();
-#pragma unroll
-                    for (int d = 0; d < 3; d++) {
-                        S.red[d][tid] = h3[d];
-                        S.red[3 + d][tid] = l3[d];
-                    }
-                    __syncthreads();
-                    if (g == 0) {
-#pragma unroll
-                        for (int d = 0; d < 3; d++) {
-                            h3[d] = l3[d] = 0.f;
-                            for (int q = 0; q < G; q++) {
-                                df_add(h3[d], l3[d], S.red[d][q * m + tt]);
-                                l3[d] += S.red[3 + d][q * m + tt];
-                            }
-                        }
-                    }
-                }
-                if (g == 0 && act) {
-                    A.nx[i] = static_cast<double>(h3[0]) + static_cast<double>(l3[0]);
-                    A.ny[i] = static_cast<double>(h3[1]) + static_cast<double>(l3[1]);
-                    A.nz[i] = static_cast<double>(h3[2]) + static_cast<double>(l3[2]);
-                }
-            } else {
-                if (G > 1) {
-                    __syncthreads();
-                    S.red[0][tid] = ax;
-                    S.red[1][tid] = ay;
-                    S.red[2][tid] = az;
-                    __syncthreads();
-                    if (g == 0) {
-                        ax = ay = az = real(0);
-                        for (int q = 0; q < G; q++) {
-                            ax += S.red[0][q * m + tt];
-                            ay += S.red[1][q * m + tt];
-                            az += S.red[2][q * m + tt];
-                        }
-                    }
-                }
-                if (g == 0 && act) {
-                    A.nx[i] = static_cast<double>(ax);
-                    A.ny[i] = static_cast<double>(ay);
-                    A.nz[i] = static_cast<double>(az);
-                }
-            }
-        }
-    }
-}
-
 // L2P of each leaf's complete local expansion (Eq. shifting at the moonlet),
 // plus the near-field sums and the external forces: one thread per moonlet
 // in tree order (the moonlets of a leaf are consecutive, so the threads of a
@@ -555,16 +371,6 @@ static void descend_t(ncorp_ctx *c, DescendArgs D) {
 }
 
 template <int P, typename real>
-static void eval_t(ncorp_ctx *c, const EvalArgs &A) {
-    int per_sm = 0;
-    NCORP_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
-        &per_sm, reinterpret_cast<const void *>(k_eval<P, real>), EV_THREADS, 0));
-    if (per_sm < 1) per_sm = 1;
-    k_eval<P, real><<<per_sm * c->num_sms, EV_THREADS, 0, c->stream>>>(A);
-    c->launches++;
-}
-
-template <int P, typename real>
 static void far_t(ncorp_ctx *c, const EvalArgs &A) {
     k_far<P, real><<<grid_for(A.n, FAR_THREADS, 8 * c->num_sms), FAR_THREADS, 0, c->stream>>>(A);
     c->launches++;
@@ -603,7 +409,6 @@ static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, double G, ExtForce
     A.gh = C.gh; A.gl = C.gl;
     A.Cf = C.Cf;
     A.Cf_lo = C.Cf_lo;
-    A.p2p_off = c->wl.p2p_off; A.p2p_src = c->wl.p2p_src; A.p2p_dir_cap = c->wl.p2p_dir_cap;
     A.x = P.x; A.y = P.y; A.z = P.z; A.m = P.m;
     A.hi4 = P.hi4; A.lo4 = P.lo4;
     A.G = G;
@@ -613,32 +418,10 @@ static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, double G, ExtForce
     A.amy = want_mutual ? c->amy : nullptr;
     A.amz = want_mutual ? c->amz : nullptr;
     A.nx = c->amx; A.ny = c->amy; A.nz = c->amz;   // the far kernel overwrites them in place
-    A.work = c->work_counter;
     A.ctl = c->ctl;
     A.kick_h = 0.0;
     A.vx = A.vy = A.vz = nullptr;
     return A;
-}
-
-// The work counter was zeroed by the gravity walk's k_walk_init.
-void launch_near(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G) {
-    const EvalArgs A = eval_args(c, P, G, ExtForce{}, false);
-#define NCORP_EVAL_CASE(PP)                      \
-    case PP:                                     \
-        if (mixed) eval_t<PP, float>(c, A);      \
-        else eval_t<PP, double>(c, A);           \
-        break;
-    switch (p) {
-        NCORP_EVAL_CASE(1)
-        NCORP_EVAL_CASE(2)
-        NCORP_EVAL_CASE(3)
-        NCORP_EVAL_CASE(4)
-        NCORP_EVAL_CASE(5)
-        NCORP_EVAL_CASE(6)
-        default: break;
-    }
-#undef NCORP_EVAL_CASE
-    NCORP_CUDA_CHECK(cudaGetLastError());
 }
 
 void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G, ExtForce ext, bool want_mutual,

@@ -175,7 +175,12 @@ void alloc_lists(ncorp_ctx *c, int front, int m2l, int p2p, int self) {
         W.p2p_dir_cap = 0;
         dalloc(W.p2p, p2p);
         dalloc(W.self, self);
+        W.near_cap = 0;
         dalloc(W.p2p_src, 2 * static_cast<size_t>(p2p) + self);   // int2
+        // at most one item per NEAR_ENTRIES_MIN entries and two more per leaf, in lists that are far from
+        // full; a tree that needs more reports it like any full list
+        dalloc(W.near_items, static_cast<size_t>(p2p) / 4 + 2 * self);
+        W.near_cap = p2p / 4 + 2 * self;
         dalloc(W.cp2p, p2p);
         dalloc(W.cself, self);
         W.p2p_cap = p2p;
@@ -642,7 +647,7 @@ void gravity(ncorp_ctx *c, ParticleSet &S, int p, double theta, double t, bool w
     NCORP_CUDA_CHECK(cudaStreamWaitEvent(c->side2, c->ev_lists, 0));
     on_stream(c, c->side2, [&] {
         Stage st(c, NCORP_STAGE_NEAR);
-        launch_near(c, S, p, mixed, G);
+        launch_near(c, S, mixed, G);
         NCORP_CUDA_CHECK(cudaEventRecord(c->ev_near, c->stream));
     });
     NCORP_CUDA_CHECK(cudaStreamWaitEvent(c->stream, c->ev_p2m, 0));
@@ -1543,7 +1548,7 @@ void ncorp_free(ncorp_ctx *c) {
         dfree(C.leaves); dfree(C.leaf_of); dfree(C.rc_spec); dfree(C.bounds); dfree(C.blocksum); dfree(C.maker); dfree(C.before); dfree(C.done);
         WalkLists &W = c->wl;
         dfree(W.front[0]); dfree(W.front[1]); dfree(W.front_count); dfree(W.m2l); dfree(W.p2p); dfree(W.self);
-        dfree(W.cnt); dfree(W.offs); dfree(W.cursor); dfree(W.m2l_dir); dfree(W.p2p_off); dfree(W.p2p_src);
+        dfree(W.cnt); dfree(W.offs); dfree(W.cursor); dfree(W.m2l_dir); dfree(W.p2p_off); dfree(W.p2p_src); dfree(W.near_items);
         dfree(W.cp2p); dfree(W.cself);
         dfree(c->ctl);
         if (c->ctl_h) cudaFreeHost(c->ctl_h);

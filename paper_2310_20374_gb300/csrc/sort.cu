@@ -900,6 +900,7 @@ struct GatherArgs {
     int *operm;
     uint32_t *oqx, *oqy, *oqz;
     float4 *hi4, *lo4;
+    double *nx, *ny, *nz;  // the near-field sums, zeroed for the kernel that adds to them
     const uint32_t *idx;
     const uint64_t *key;   // sorted keys
     const unsigned short *disk_of;   // a forest: disk of each position (equal keys of two disks are no run)
@@ -943,6 +944,9 @@ __global__ void k_gather(GatherArgs g) {
         g.oqx[d] = g.qx[j];
         g.oqy[d] = g.qy[j];
         g.oqz[d] = g.qz[j];
+        g.nx[i] = 0.0;
+        g.ny[i] = 0.0;
+        g.nz[i] = 0.0;
         // double-float copy of the position: x = hi + lo with both parts FP32
         const double X = g.x[j], Y = g.y[j], Z = g.z[j];
         const float hx = static_cast<float>(X), hy = static_cast<float>(Y), hz = static_cast<float>(Z);
@@ -974,6 +978,7 @@ void launch_gather(ncorp_ctx *c, const ParticleSet &src_xv, const ParticleSet &s
     g.om = dst.m; g.oR = dst.R; g.operm = dst.perm;
     g.oqx = dst.qx; g.oqy = dst.qy; g.oqz = dst.qz;
     g.hi4 = dst.hi4; g.lo4 = dst.lo4;
+    g.nx = c->amx; g.ny = c->amy; g.nz = c->amz;
     g.idx = idx;
     g.key = dst.key;
     g.disk_of = c->nd > 1 ? c->disk_of : nullptr;

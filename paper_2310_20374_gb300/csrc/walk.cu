@@ -53,6 +53,8 @@ struct WalkArgs {
     // per-target lists (gravity): counting sort by target cell
     int *cnt, *offs, *cursor, *p2p_off;
     int2 *p2p_src;             // per directed near-field entry: the source leaf's (first, count)
+    int4 *near_items;          // near-field work items (count ctl->n_near)
+    int near_cap;
     const int *first;
     int2 *m2l_dir;
     int m2l_dir_cap, p2p_dir_cap;
@@ -88,6 +90,7 @@ __global__ void k_walk_init(WalkArgs A) {
     A.ctl->n_m2l = 0;
     A.ctl->n_p2p = 0;
     A.ctl->n_self = 0;
+    A.ctl->n_near = 0;
     A.ctl->dec_pairs = 0;
     A.ctl->dec_self = 0;
     A.ctl->n_inter = 0;
@@ -195,6 +198,8 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
     }
     if (!grid_sync(A.ctl, bar)) return;
     {
+        __shared__ int s_items;
+        const int n_leaves = A.ctl->n_leaves;
         int pm = 0, pp = 0;
         for (int b = threadIdx.x; b < static_cast<int>(blockIdx.x); b += blockDim.x) {
             pm += __ldcg(&bs[b]);
@@ -213,6 +218,29 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
                 A.cursor[i] = pm + xm;
                 A.p2p_off[i] = pp + xp;   // direct: offsets (in place), cursors in cnt
                 A.cnt[i] = pp + xp;
+            }
+            // the near field's items: a subset of the leaf's moonlets and an equal share of its entries each
+            const int m = vp > 0 ? __ldg(&A.count[i]) : 0;
+            int parts = 0;
+            for (int t = 0; t < m; t += near_targets(m - t)) parts += near_shares(vp, near_targets(m - t), n_leaves);
+            int total_items = 0;
+            const int xi = block_prefix(parts, s_tmp, &total_items);
+            if (threadIdx.x == 0) s_items = total_items ? atomicAdd(&A.ctl->n_near, total_items) : 0;
+            __syncthreads();
+            if (parts > 0) {
+                const int f = __ldg(&A.first[i]), s0 = pp + xp;
+                int slot = s_items + xi;
+                if (slot + parts > A.near_cap || s0 + vp > A.p2p_dir_cap) {
+                    atomicOr(&A.ctl->err, ERR_DIRECTED);
+                } else {
+                    for (int t = 0; t < m; t += near_targets(m - t)) {
+                        const int k = near_targets(m - t), np = near_shares(vp, k, n_leaves);
+                        for (int q = 0; q < np; q++)
+                            A.near_items[slot++] = make_int4(f + t, np == 1 ? k : -k,
+                                                             s0 + static_cast<int>(static_cast<long long>(vp) * q / np),
+                                                             s0 + static_cast<int>(static_cast<long long>(vp) * (q + 1) / np));
+                    }
+                }
             }
             pm += sm;
             pp += sp;
@@ -625,6 +653,7 @@ void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     A.cp2p = W.cp2p; A.cp2p_cap = W.p2p_cap;
     A.cself = W.cself; A.cself_cap = W.self_cap;
     A.cnt = W.cnt; A.offs = W.offs; A.cursor = W.cursor; A.p2p_off = W.p2p_off; A.p2p_src = W.p2p_src;
+    A.near_items = W.near_items; A.near_cap = W.near_cap;
     A.m2l_dir = W.m2l_dir; A.m2l_dir_cap = W.m2l_dir_cap; A.p2p_dir_cap = W.p2p_dir_cap;
     A.work = gravity ? c->work_counter : nullptr;
     A.ctl = c->ctl;
