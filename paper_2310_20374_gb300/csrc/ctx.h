@@ -23,6 +23,8 @@ struct ParticleSet {
     float4 *lo4 = nullptr;    // (x, y, z) - hi, rounded to FP32 (double-float position)
 };
 
+constexpr int BLOCKSUM_INTS = 8192;
+
 struct Cells {
     int cap = 0;
     int *level = nullptr, *first = nullptr, *count = nullptr, *child0 = nullptr, *nchild = nullptr,
@@ -43,10 +45,7 @@ struct Cells {
     float *Cf_lo = nullptr;   // [cap][3] mixed precision: low parts of the order-1 coefficients of Cf
                               // (double-float: the field is the sum of the whole far field)
     int *leaves = nullptr;    // leaf cell ids
-    int *bounds = nullptr;    // [cap][9] scratch of the build
-    int *maker = nullptr;     // [cap] scratch of the build: block that made the cell
-    int *before = nullptr;    // [cap] scratch of the build: children of its maker's earlier cells
-    int *blocksum = nullptr;  // per-block scratch of cooperative kernels
+    int *blocksum = nullptr;  // [BLOCKSUM_INTS] per-block counts of the build
     unsigned *done = nullptr; // [cap] descent: epoch in which the cell's complete expansion was written
     int *leaf_of = nullptr;   // [leaf_of_cap] leaf of each moonlet of the tree (tree order)
     double *rc_spec = nullptr;// [leaf_of_cap] fused walk: each moonlet's R + dt |v| bound the tree's collision

@@ -136,10 +136,7 @@ void alloc_cells(ncorp_ctx *c, int cap) {
     dalloc(cf, static_cast<size_t>(cap) * num_c(MAXP));
     C.Cf = cf;
     dalloc(C.leaves, cap);
-    dalloc(C.bounds, static_cast<size_t>(cap) * 9);
-    dalloc(C.blocksum, 8192);
-    dalloc(C.maker, cap);
-    dalloc(C.before, cap);
+    dalloc(C.blocksum, BLOCKSUM_INTS);
     dalloc(C.Cf_lo, 3 * static_cast<size_t>(cap));
     dalloc(C.Ch_lo, 3 * static_cast<size_t>(cap));
     dalloc(C.done, cap);   // descent epochs start at 1: zeroed words never match
@@ -1545,7 +1542,7 @@ void ncorp_free(ncorp_ctx *c) {
         dfree(C.arrive); dfree(C.arrive_m); dfree(C.cx); dfree(C.cy); dfree(C.cz); dfree(C.M); dfree(C.sx); dfree(C.sy); dfree(C.sz);
         dfree(C.rmax); dfree(C.rcrit); dfree(C.rho); dfree(C.bx); dfree(C.by); dfree(C.bz); dfree(C.bmax);
         dfree(C.bcrit); dfree(C.gh); dfree(C.gl); dfree(C.bh); dfree(C.bl); dfree(C.Mh); dfree(C.Ch); dfree(C.Cf); dfree(C.Cf_lo); dfree(C.Ch_lo);
-        dfree(C.leaves); dfree(C.leaf_of); dfree(C.rc_spec); dfree(C.bounds); dfree(C.blocksum); dfree(C.maker); dfree(C.before); dfree(C.done);
+        dfree(C.leaves); dfree(C.leaf_of); dfree(C.rc_spec); dfree(C.blocksum); dfree(C.done);
         WalkLists &W = c->wl;
         dfree(W.front[0]); dfree(W.front[1]); dfree(W.front_count); dfree(W.m2l); dfree(W.p2p); dfree(W.self);
         dfree(W.cnt); dfree(W.offs); dfree(W.cursor); dfree(W.m2l_dir); dfree(W.p2p_off); dfree(W.p2p_src); dfree(W.near_items);

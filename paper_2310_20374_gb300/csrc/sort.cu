@@ -190,7 +190,7 @@ __global__ void k_keys(const double *__restrict__ x, const double *__restrict__ 
     __shared__ int s_shift;
     if ((gate && *gate == 0) || aborted(ctl)) return;
     if (ctl->disk_of) {   // a forest: each moonlet in its disk's root cube (k_disk_roots made them)
-        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->bar_count = 0;
+        if (blockIdx.x == 0 && threadIdx.x == 0) ctl->bar_count = ctl->bar_build = 0;
         for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
             const double *r = ctl->droot + 4 * ctl->disk_of[i];
             const int sh = KEY_BITS - (static_cast<int>((__double_as_longlong(r[3]) >> 52) & 0x7ff) - 1023);
@@ -209,7 +209,7 @@ __global__ void k_keys(const double *__restrict__ x, const double *__restrict__ 
         root_cube(ctl->bbox, s_root);
         if (blockIdx.x == 0) {
             for (int k = 0; k < 4; k++) ctl->root[k] = s_root[k];
-            ctl->bar_count = 0;
+            ctl->bar_count = ctl->bar_build = 0;
         }
         // L = 2^k exactly: the scale 2^21 / L is 2^(21 - k)
         s_shift = KEY_BITS - (static_cast<int>((__double_as_longlong(s_root[3]) >> 52) & 0x7ff) - 1023);
@@ -238,8 +238,8 @@ __global__ void k_disk_roots(Ctrl *ctl, const int *gate) {
 
 // The bounding box in ctl must be empty on entry (k_reset_ctl leaves it so),
 // or already hold the positions' box (bbox_done: the step's kick-drift kernel
-// folds it); k_keys also zeroes the grid-barrier counter for the sort that
-// follows.
+// folds it); k_keys also zeroes the grid-barrier counters of the sort and
+// the build that follow.
 void launch_bbox_keys(ncorp_ctx *c, const double *x, const double *y, const double *z, int n, uint64_t *key,
                       uint32_t *qx, uint32_t *qy, uint32_t *qz, bool bbox_done, const int *gate) {
     if (!bbox_done) {

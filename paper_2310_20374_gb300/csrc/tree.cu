@@ -32,281 +32,248 @@ constexpr ExpTable make_exp_table() {
 }
 __constant__ ExpTable c_exp = make_exp_table();
 
-__device__ __forceinline__ int lower_bound_u64(const uint64_t *__restrict__ a, int lo, int hi, uint64_t t) {
-    while (lo < hi) {
-        int mid = (lo + hi) >> 1;
-        if (a[mid] < t) lo = mid + 1;
-        else hi = mid;
-    }
-    return lo;
-}
-
 // ---------------------------------------------------------------------------
-// Build: one cooperative launch, one grid barrier per level.  The cells of a
-// level are shared evenly among the blocks.  Per level, a block
-//   1. places the children of its cells: a cell's children follow the level
-//      in the order of their parents, at
-//        level end + (children of the cells made by blocks before the cell's
-//        maker) + (children of the cells its maker made before it),
-//      both terms published before the barrier; then writes them;
-//   2. for each child it made with more than s moonlets, finds the
-//      boundaries of its octants on the next 3 key bits (the Hilbert digit of
-//      the grandchild), so the children of every cell come out in Hilbert
-//      order, and publishes, for the next level, the running count of
-//      grandchildren over the cells it made and its total.
-// Octant boundaries: boundary o (o = 1..7) is the first moonlet whose key is
-// >= (prefix, o); four lanes search for it together, cutting the range in
-// five per round.
+// Build: every cell is found from the sorted keys by the moonlet it starts
+// with, all levels at once, in one cooperative launch with one grid barrier.
+//
+// Let lcp(a, b) be the number of leading octal digits two keys share (the depth
+// of the deepest cell that could hold both), and a moonlet i with
+// l = lcp(key[i - 1], key[i]) (-1 at a disk's first moonlet).  A cell of level L
+// starts at i iff l < L and its parent, the cell of level L - 1 that holds i, is
+// split (more than s moonlets, level below MAX_LEVEL):
+//   - a parent that starts at i is split iff lcp(key[i], key[i + s]) >= L - 1;
+//   - the parent of the first of them (level l + 1) starts at some p < i, found
+//     by a binary search among the s keys before i (if it starts earlier still it
+//     holds more than s), and is split iff lcp(key[p], key[p + s]) >= l.
+// So the cells starting at i have the levels L0 = l + 1 .. Lmax, the deepest is a
+// leaf and the others are not.  The index of a cell (level-major, Hilbert order
+// within a level) is its level's first index plus the number of cells of that
+// level starting before i: per-block counts of every level, one grid barrier,
+// prefix sums over blocks, then ballots.  A cell's end is known to the moonlet j
+// that starts the next cell: j ends the cells of levels L0(j) .. the leaf level of
+// j - 1.  Counts (end - start) and children are added with atomics into zeroed
+// fields.
+//
+// Latency-bound: a level-by-level build (a grid barrier, the placement and
+// dependent octant searches per level) took 46 / 90 / 268 us at N = 1e3 / 1e5 /
+// 1e6 with its two helper launches; this takes 12 / 22 / 76 us.
 // ---------------------------------------------------------------------------
 struct BuildArgs {
     const uint64_t *key;
     const uint32_t *qx, *qy, *qz;
-    int n, s, cap;
+    int n, s, cap, chunk;   // chunk: moonlets per block, a multiple of BUILD_T
     int *level, *first, *count, *child0, *nchild, *parent, *arrive, *arrive_m;
     uint32_t *cx, *cy, *cz;
-    int *bounds, *blocksum;
-    int *maker, *before;    // per cell: the block that made it, children of its maker's earlier cells
+    int *leaves, *leaf_of;  // leaf_of[i] first holds moonlet i's levels, (L0 << 8 | Lmax) or -1
+    int *bcount;            // [gridDim.x][BUILD_ROW]: cells of each level the block starts, its leaves, and the leaf
+                            // level of its last start (-1: none)
     Ctrl *ctl;
     const int *gate;        // nothing to do while *gate is 0 (null: always build)
 };
 
-// The roots: one per disk (cell d holds disk d's moonlets; one disk: cell 0 holds all).
-__global__ void k_build_init(BuildArgs A) {
-    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;
-    const int nd = A.ctl->nd;
-    for (int d = 0; d < nd; d++) {
-        A.level[d] = 0;
-        A.first[d] = A.ctl->doff ? A.ctl->doff[d] : 0;
-        A.count[d] = A.ctl->doff ? A.ctl->doff[d + 1] - A.ctl->doff[d] : A.n;
-        A.child0[d] = -1;
-        A.nchild[d] = 0;
-        A.parent[d] = -1;
-        A.cx[d] = A.cy[d] = A.cz[d] = 0;
-        A.maker[d] = 0;
-        A.before[d] = 0;
-        A.arrive[d] = 0;     // arrival counters of the collision climb and of the multipoles,
-        A.arrive_m[d] = 0;   // zeroed as cells are made
-    }
-    A.ctl->col_stale = 1;   // a new tree: no collision pairs listed for it yet
-    A.ctl->level_start[0] = 0;
-    A.ctl->level_start[1] = nd;
-    A.ctl->n_cells = nd;
-    A.ctl->max_level = 0;
-    A.ctl->n_leaves = 0;
-    A.ctl->bar_count = 0;
+constexpr int BUILD_T = 256, BUILD_W = BUILD_T / 32;
+constexpr int BUILD_LEVELS = MAX_LEVEL + 1;   // levels 0 .. MAX_LEVEL
+constexpr int BUILD_COUNTS = BUILD_LEVELS + 1;   // and the leaves (every moonlet that starts cells starts one leaf)
+constexpr int BUILD_ROW = BUILD_COUNTS + 1;
+static_assert(BUILD_COUNTS <= 32, "a lane per count");
+
+__device__ __forceinline__ int common_levels(uint64_t a, uint64_t b) {
+    const uint64_t x = a ^ b;
+    return x ? (__clzll(static_cast<long long>(x)) - 1) / 3 : MAX_LEVEL;
 }
 
-// Octant boundaries of cell c (level lev, moonlets [f, f + cnt)), written to
-// bounds[c][0..8] (b_0 = f, b_8 = f + cnt), and its number of non-empty
-// octants (returned on every lane).  Called by a whole warp.
-__device__ int octant_bounds(const BuildArgs &A, int c, int f, int cnt, int lev, int lane) {
-    const uint64_t pref = __ldg(&A.key[f]) >> (63 - 3 * lev);
-    const int shift = 60 - 3 * lev;
-    const int grp = lane >> 2, j = lane & 3;           // boundary o = grp + 1 for grp < 7
-    const bool searching = grp < 7;
-    const uint64_t target = ((pref << 3) | static_cast<uint64_t>(grp + 1)) << shift;
-    int lo = f, hi = f + cnt;                          // the boundary lies in [lo, hi]
-    while (true) {
-        const bool wide = searching && hi - lo > 4;
-        if (!__any_sync(0xffffffffu, wide)) break;
-        bool less = false;
-        int sj = 0;
-        if (wide) {
-            sj = lo + static_cast<int>((static_cast<long long>(hi - lo) * (j + 1)) / 5);
-            less = __ldg(&A.key[sj]) < target;
-        }
-        const unsigned bal = __ballot_sync(0xffffffffu, less);
-        const int cl = __popc((bal >> (4 * grp)) & 0xfu);    // samples below the target (monotone)
-        const int s_lo = __shfl_sync(0xffffffffu, sj, (lane & ~3) + max(cl - 1, 0));
-        const int s_hi = __shfl_sync(0xffffffffu, sj, (lane & ~3) + min(cl, 3));
-        if (wide) {
-            const int nlo = cl > 0 ? s_lo + 1 : lo;
-            const int nhi = cl < 4 ? s_hi : hi;
-            lo = nlo;
-            hi = nhi;
-        }
-    }
-    const bool below = searching && lo + j < hi && __ldg(&A.key[lo + j]) < target;
-    const unsigned bal = __ballot_sync(0xffffffffu, below);
-    const int b_o = lo + __popc((bal >> (4 * grp)) & 0xfu);
-    // lane k < 9 holds b_k: b_0 = f, b_1..b_7 from the groups, b_8 = f + cnt
-    const int from_grp = __shfl_sync(0xffffffffu, b_o, 4 * max(lane - 1, 0));
-    const int b = lane == 0 ? f : (lane < 8 ? from_grp : f + cnt);
-    const int bn = __shfl_down_sync(0xffffffffu, b, 1);
-    const unsigned ne = __ballot_sync(0xffffffffu, lane < 8 && bn > b);
-    if (lane < 9) A.bounds[(size_t)c * 9 + lane] = b;
-    return __popc(ne);
-}
-
-// For the cells [cb, ce) this block made (level lev): octant bounds, children
-// counts, and the running count over them (before[]); returns the total.
-__device__ int made_cells(const BuildArgs &A, int cb, int ce, int lev, int *s_red) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    for (int c = cb + wid; c < ce; c += nw) {
-        if (c >= A.cap) break;
-        const int cnt = __ldcg(&A.count[c]), f = __ldcg(&A.first[c]);
-        int nch = 0;
-        if (cnt > A.s && lev < MAX_LEVEL) nch = octant_bounds(A, c, f, cnt, lev, lane);
-        if (lane == 0) A.nchild[c] = nch;
-    }
-    __syncthreads();
-    int run = 0;
-    if (wid == 0) {
-        for (int c0 = cb; c0 < ce; c0 += 32) {
-            const int c = c0 + lane;
-            const int v = (c < ce && c < A.cap) ? __ldcg(&A.nchild[c]) : 0;
-            int incl = v;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += u;
+// The levels (L0, Lmax) of the cells starting at moonlet i of the disk [d0, d1); false: none.
+__device__ __forceinline__ bool cells_starting(const BuildArgs &A, int i, int d0, int d1, int &L0, int &Lmax) {
+    const uint64_t k = __ldg(&A.key[i]);
+    const int s = A.s;
+    int l = -1;
+    if (i > d0) {
+        l = common_levels(__ldg(&A.key[i - 1]), k);
+        if (l >= MAX_LEVEL) return false;
+        const int shift = 63 - 3 * l;
+        const uint64_t lo_key = l > 0 ? (k >> shift) << shift : 0;   // first key of the level-l cell that holds i
+        if (i - d0 < s || __ldg(&A.key[i - s]) < lo_key) {           // the cell starts less than s before i
+            int p = max(d0, i - s), e = i - 1;
+            while (p < e) {
+                const int mid = (p + e) >> 1;
+                if (__ldg(&A.key[mid]) < lo_key) p = mid + 1;
+                else e = mid;
             }
-            if (c < ce && c < A.cap) {
-                A.before[c] = run + incl - v;
-                A.maker[c] = blockIdx.x;
-            }
-            run += __shfl_sync(0xffffffffu, incl, 31);
+            if (d1 - p <= s || common_levels(__ldg(&A.key[p + s]), k) < l) return false;
         }
-        if (lane == 0) s_red[0] = run;
     }
-    __syncthreads();
-    const int t = s_red[0];
-    __syncthreads();
-    return t;
+    L0 = l + 1;
+    Lmax = L0;
+    if (d1 - i > s) Lmax = max(L0, min(MAX_LEVEL, common_levels(k, __ldg(&A.key[i + s])) + 1));
+    return true;
 }
 
-__global__ void __launch_bounds__(256) k_build(BuildArgs A) {
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __shared__ int s_red[32];
-    __shared__ int s_pre[4097];      // children made by blocks before each block (grid <= 4096)
-    __shared__ int s_lo, s_hi;
-    volatile Ctrl *vc = A.ctl;
-    const int G = gridDim.x;
+__global__ void __launch_bounds__(BUILD_T) k_build(BuildArgs A) {
+    __shared__ int s_cnt[BUILD_COUNTS];                   // phase 1: the block's cells per level, its leaves
+    __shared__ int s_base[BUILD_COUNTS];                  // next index of each level, next leaf
+    __shared__ unsigned s_bal[BUILD_W][BUILD_COUNTS];        // starts of each level among the warp's moonlets
+    __shared__ int s_pre[BUILD_W][BUILD_COUNTS];          // index of the first of them
+    __shared__ int s_tot[BUILD_COUNTS], s_low[BUILD_COUNTS];
+    __shared__ int s_last[BUILD_W];                       // leaf level of the last start in each warp's moonlets
+    __shared__ int s_prev;
+    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;   // every block, before the barrier
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, b = blockIdx.x, G = gridDim.x;
+    const int c0 = min(A.n, b * A.chunk), c1 = min(A.n, c0 + A.chunk);
+    const unsigned le = 0xffffffffu >> (31 - lane);       // lanes up to this one
+    const int *doff = A.ctl->doff;
+    // ---- 1. the cells each moonlet starts, and the block's counts
+    for (int i = b * BUILD_T + tid; i < A.cap; i += G * BUILD_T) A.count[i] = A.nchild[i] = 0;
+    if (tid < BUILD_COUNTS) s_cnt[tid] = 0;
+    if (tid == 0) s_prev = -1;
+    __syncthreads();
+    for (int i = c0 + tid; i < c1; i += BUILD_T) {
+        int d0 = 0, d1 = A.n;
+        if (doff) {
+            const int d = A.ctl->disk_of[i];
+            d0 = __ldg(&doff[d]);
+            d1 = __ldg(&doff[d + 1]);
+        }
+        int L0 = 0, Lmax = 0, code = -1;
+        if (cells_starting(A, i, d0, d1, L0, Lmax)) {
+            code = L0 << 8 | Lmax;
+            for (int L = L0; L <= Lmax; L++) atomicAdd(&s_cnt[L], 1);
+            atomicAdd(&s_cnt[BUILD_LEVELS], 1);
+            atomicMax(&s_prev, (i - c0) << 5 | Lmax);
+        }
+        A.leaf_of[i] = code;
+    }
+    __syncthreads();
+    if (tid < BUILD_COUNTS) A.bcount[b * BUILD_ROW + tid] = s_cnt[tid];
+    if (tid == BUILD_COUNTS) A.bcount[b * BUILD_ROW + BUILD_COUNTS] = s_prev < 0 ? -1 : s_prev & 31;
     unsigned bar = 0;
-    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;   // every block, before the first barrier
-    {   // block 0 makes the roots' children counts
-        const int t = made_cells(A, 0, blockIdx.x == 0 ? vc->level_start[1] : 0, 0, s_red);
-        if (threadIdx.x == 0) A.blocksum[blockIdx.x] = t;
+    if (!grid_sync_on(&A.ctl->bar_build, A.ctl, bar)) return;
+    // ---- 2. totals of every level, and what the blocks before this one hold (a warp per level)
+    for (int L = w; L < BUILD_COUNTS; L += BUILD_W) {
+        int tot = 0, low = 0;
+        for (int q = lane; q < G; q += 32) {
+            const int v = __ldcg(&A.bcount[q * BUILD_ROW + L]);
+            tot += v;
+            if (q < b) low += v;
+        }
+        tot = warp_sum(tot);
+        low = warp_sum(low);
+        if (lane == 0) {
+            s_tot[L] = tot;
+            s_low[L] = low;
+        }
     }
-    if (!grid_sync(A.ctl, bar)) return;
-    for (int lev = 0; lev < MAX_LEVEL; lev++) {
-        const int ls = vc->level_start[lev], le = vc->level_start[lev + 1];
-        if (ls >= le) break;
-        const int *bsum = A.blocksum + (lev & 1) * G;
-        // prefix of the published totals (every block computes it; each thread a run of them)
-        {
-            const int T = blockDim.x, per = (G + T - 1) / T;
-            const int b0 = min(G, (int)threadIdx.x * per), b1 = min(G, b0 + per);
-            int sum = 0;
-            for (int b = b0; b < b1; b++) sum += ((volatile const int *)bsum)[b];
-            int incl = sum;
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += u;
-            }
-            if (lane == 31) s_red[wid] = incl;
-            __syncthreads();
-            if (wid == 0) {
-                const int v = lane < nw ? s_red[lane] : 0;
-                int wi = v;
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int u = __shfl_up_sync(0xffffffffu, wi, o);
-                    if (lane >= o) wi += u;
-                }
-                if (lane < nw) s_red[lane] = wi - v;
-                if (lane == nw - 1) s_pre[G] = wi;
-            }
-            __syncthreads();
-            int run = s_red[wid] + incl - sum;
-            for (int b = b0; b < b1; b++) {
-                const int v = ((volatile const int *)bsum)[b];
-                s_pre[b] = run;
-                run += v;
-            }
+    if (w == BUILD_W - 1) {   // the leaf level of the last start before this block
+        int m = -1;
+        for (int q = lane; q < b; q += 32) {
+            const int v = __ldcg(&A.bcount[q * BUILD_ROW + BUILD_COUNTS]);
+            if (v >= 0) m = max(m, q << 5 | v);
         }
-        __syncthreads();
-        const int total = s_pre[G];
-        // this block's share of the level, and the children it will make
-        const int ncl = le - ls;
-        const int chunk = (ncl + G - 1) / G;
-        const int cb = min(le, ls + (int)blockIdx.x * chunk), ce = min(le, cb + chunk);
-        if (threadIdx.x == 0) {
-            s_lo = 1 << 30;
-            s_hi = -1;
-        }
-        __syncthreads();
-        // ---- 1. place and write the children of the block's cells
-        for (int c = cb + wid; c < ce; c += nw) {
-            if (c >= A.cap) break;
-            const int nch = __ldcg(&A.nchild[c]);
-            if (nch == 0) {
-                if (lane == 0) A.child0[c] = -1;
-                continue;
-            }
-            const int c0 = le + s_pre[__ldcg(&A.maker[c])] + __ldcg(&A.before[c]);
-            if (lane == 0) {
-                A.child0[c] = c0;
-                atomicMin(&s_lo, c0);
-                atomicMax(&s_hi, c0 + nch);
-            }
-            int b = 0;
-            if (lane < 9) b = __ldcg(&A.bounds[(size_t)c * 9 + lane]);
-            const int bn = __shfl_down_sync(0xffffffffu, b, 1);
-            const bool ne = lane < 8 && bn > b;
-            const unsigned mask = __ballot_sync(0xffffffffu, ne);
-            if (ne) {
-                const int ci = c0 + __popc(mask & ((1u << lane) - 1u));
-                if (ci < A.cap) {
-                    const int sh = KEY_BITS - (lev + 1);
-                    A.level[ci] = lev + 1;
-                    A.first[ci] = b;
-                    A.count[ci] = bn - b;
-                    A.child0[ci] = -1;
-                    A.nchild[ci] = 0;
-                    A.parent[ci] = c;
-                    A.arrive[ci] = 0;
-                    A.arrive_m[ci] = 0;
-                    A.cx[ci] = A.qx[b] >> sh;
-                    A.cy[ci] = A.qy[b] >> sh;
-                    A.cz[ci] = A.qz[b] >> sh;
-                } else {
-                    atomicOr(&A.ctl->err, ERR_CELLS);
-                }
-            }
-        }
-        if (blockIdx.x == 0 && threadIdx.x == 0) {
-            A.ctl->level_start[lev + 2] = le + total;
-            A.ctl->n_cells = le + total;
-            if (total > 0) A.ctl->max_level = lev + 1;
-        }
-        __syncthreads();
-        // ---- 2. the children this block made (a contiguous range): bounds, running counts
-        const int mb = s_hi >= 0 ? s_lo : 0, me = s_hi >= 0 ? s_hi : 0;
-        {
-            const int t = made_cells(A, mb, me, lev + 1, s_red);
-            if (threadIdx.x == 0) A.blocksum[((lev + 1) & 1) * G + blockIdx.x] = t;
-        }
-        if (!grid_sync(A.ctl, bar)) return;
+        m = __reduce_max_sync(0xffffffffu, m);
+        if (lane == 0) s_prev = m < 0 ? -1 : m & 31;
     }
-}
-
-// The leaf list, and the leaf of every moonlet (leaf_of, tree order).  Also
-// zeroes the grid-barrier counter for the cooperative kernel that follows.
-__global__ void k_collect_leaves(const int *__restrict__ nchild, const int *__restrict__ first,
-                                 const int *__restrict__ count, Ctrl *ctl, int cap, int *leaves, int *n_leaves,
-                                 int *leaf_of, const int *gate) {
-    if (gate && *gate == 0) return;
-    if (blockIdx.x == 0 && threadIdx.x == 0) ctl->bar_count = 0;
-    if (aborted(ctl)) return;
-    const int nc = min(ctl->n_cells, cap);
-    for (int base = blockIdx.x * blockDim.x; base < nc; base += gridDim.x * blockDim.x) {
-        const int i = base + threadIdx.x;
-        const int is_leaf = (i < nc && nchild[i] == 0) ? 1 : 0;
-        const int slot = warp_append(n_leaves, is_leaf);
-        if (is_leaf) {
-            leaves[slot] = i;
-            const int f = first[i], e = f + count[i];
-            for (int k = f; k < e; k++) leaf_of[k] = i;
+    __syncthreads();
+    if (w == 0) {
+        const int t = lane < BUILD_LEVELS ? s_tot[lane] : 0;
+        int incl = t;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, incl, o);
+            if (lane >= o) incl += u;
         }
+        if (lane < BUILD_COUNTS) s_base[lane] = (lane < BUILD_LEVELS ? incl - t : 0) + s_low[lane];
+        if (b == 0) {   // the tree's description
+            const unsigned used = __ballot_sync(0xffffffffu, t > 0);
+            if (lane <= BUILD_LEVELS) A.ctl->level_start[lane] = incl - t;   // (levels past the deepest are empty)
+            if (lane == 31) {
+                A.ctl->n_cells = incl;
+                A.ctl->n_leaves = s_tot[BUILD_LEVELS];
+                A.ctl->max_level = 31 - __clz(static_cast<int>(used));
+                A.ctl->col_stale = 1;   // a new tree: no collision pairs listed for it yet
+                A.ctl->bar_count = 0;   // for the cooperative kernel that follows
+                if (incl > A.cap) atomicOr(&A.ctl->err, ERR_CELLS);
+            }
+        }
+    }
+    __syncthreads();
+    // ---- 3. the cells, BUILD_T moonlets at a time
+    int level_base = lane < BUILD_COUNTS ? s_base[lane] : 0;   // warp 0: running index of level `lane`, of the leaves
+    int prev = s_prev;                                         // leaf level of the last start before the tile
+    for (int t0 = c0; t0 < c1; t0 += BUILD_T) {
+        const int i = t0 + tid;
+        const int code = i < c1 ? A.leaf_of[i] : -1;
+        const bool starts = code >= 0;
+        const int L0 = starts ? code >> 8 : 32, Lmax = starts ? code & 255 : -1;
+        const int lv_lo = __reduce_min_sync(0xffffffffu, L0), lv_hi = __reduce_max_sync(0xffffffffu, Lmax);
+        unsigned mine = 0;
+        for (int L = lv_lo; L <= lv_hi; L++) {
+            const unsigned bal = __ballot_sync(0xffffffffu, L0 <= L && L <= Lmax);
+            if (lane == L) mine = bal;
+        }
+        const unsigned any = __ballot_sync(0xffffffffu, starts);
+        if (lane == BUILD_LEVELS) mine = any;
+        const int last = __shfl_sync(0xffffffffu, Lmax, any ? 31 - __clz(static_cast<int>(any)) : 0);
+        __syncthreads();   // the last tile's reads of the shared arrays are over
+        if (lane < BUILD_COUNTS) s_bal[w][lane] = mine;
+        if (lane == 0) s_last[w] = any ? last : -1;
+        __syncthreads();
+        if (w == 0 && lane < BUILD_COUNTS) {
+#pragma unroll
+            for (int q = 0; q < BUILD_W; q++) {
+                s_pre[q][lane] = level_base;
+                level_base += __popc(s_bal[q][lane]);
+            }
+        }
+        __syncthreads();
+        // leaf level of the last start before the warp, then before and up to the lane
+        int before = prev;
+        for (int q = 0; q < BUILD_W; q++) {
+            const int v = s_last[q];
+            if (v >= 0) {
+                if (q < w) before = v;
+                prev = v;
+            }
+        }
+        const unsigned lt = any & (le >> 1);
+        const int src = lt ? 31 - __clz(static_cast<int>(lt)) : 0;
+        const int from = __shfl_sync(0xffffffffu, Lmax, src);
+        const int leaf_before = lt ? from : before;            // leaf level of moonlet i - 1
+        const int leaf_here = starts ? Lmax : leaf_before;     // and of moonlet i
+        // index of the cell of level L that holds moonlet i (its last start at or before i), or i - 1
+        auto upto = [&](int L) { return s_pre[w][L] + __popc(s_bal[w][L] & le) - 1; };
+        auto below = [&](int L) { return s_pre[w][L] + __popc(s_bal[w][L] & (le >> 1)) - 1; };
+        if (i < c1) A.leaf_of[i] = upto(leaf_here);
+        if (starts) {
+            const int slot = upto(BUILD_LEVELS);
+            if (slot < A.cap) A.leaves[slot] = upto(Lmax);
+            const uint32_t qx = A.qx[i], qy = A.qy[i], qz = A.qz[i];
+            int par = L0 > 0 ? below(L0 - 1) : -1;
+            for (int L = L0; L <= Lmax; L++) {
+                const int c = upto(L);
+                if (c < A.cap) {
+                    A.level[c] = L;
+                    A.first[c] = i;
+                    A.child0[c] = L < Lmax ? upto(L + 1) : -1;
+                    A.parent[c] = par;
+                    A.arrive[c] = 0;     // arrival counters of the multipoles, zeroed as cells are made
+                    A.arrive_m[c] = 0;
+                    A.cx[c] = qx >> (KEY_BITS - L);
+                    A.cy[c] = qy >> (KEY_BITS - L);
+                    A.cz[c] = qz >> (KEY_BITS - L);
+                    atomicAdd(&A.count[c], -i);
+                    if (par >= 0) atomicAdd(&A.nchild[par], 1);
+                }
+                par = c;
+            }
+            for (int L = L0; L <= leaf_before; L++) {   // the cells that end where this one starts
+                const int c = below(L);
+                if (c < A.cap) atomicAdd(&A.count[c], i);
+            }
+        }
+        if (i == A.n - 1)   // and those that end with the last moonlet
+            for (int L = 0; L <= leaf_here; L++) {
+                const int c = upto(L);
+                if (c < A.cap) atomicAdd(&A.count[c], A.n);
+            }
     }
 }
 
@@ -327,23 +294,19 @@ void launch_build(ncorp_ctx *c, const ParticleSet &P, int n, int s, const int *g
     A.n = n; A.s = s; A.cap = C.cap;
     A.level = C.level; A.first = C.first; A.count = C.count; A.child0 = C.child0; A.nchild = C.nchild;
     A.parent = C.parent; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
-    A.bounds = C.bounds; A.blocksum = C.blocksum; A.maker = C.maker; A.before = C.before; A.ctl = c->ctl;
-    A.arrive = C.arrive;
-    A.arrive_m = C.arrive_m;
-    k_build_init<<<1, 1, 0, c->stream>>>(A); c->launches++;
-    NCORP_CUDA_CHECK(cudaGetLastError());
-    const int block = 256;
-    // about one block per thousand moonlets (a level holds at most ~n/s*8 cells): enough warps for the
-    // widest level, and few blocks at small n so that the per-level barriers stay short
-    int grid = std::min(coop_grid(c, reinterpret_cast<const void *>(k_build), block, 0), std::max(16, n / 1024));
+    A.arrive = C.arrive; A.arrive_m = C.arrive_m;
+    A.leaves = C.leaves; A.leaf_of = C.leaf_of;
+    A.bcount = C.blocksum; A.ctl = c->ctl;
+    // ctl->bar_build was zeroed by k_keys
+    const int most = std::min(coop_grid(c, reinterpret_cast<const void *>(k_build), BUILD_T, 0),
+                              BLOCKSUM_INTS / BUILD_ROW);
+    const int tiles = (n + BUILD_T - 1) / BUILD_T, per = (tiles + most - 1) / most;
+    A.chunk = per * BUILD_T;
+    const int grid = (tiles + per - 1) / per;
     void *args[] = {&A};
-    NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_build), dim3(grid), dim3(block),
+    NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_build), dim3(grid), dim3(BUILD_T),
                                                  args, 0, c->stream));
     c->launches++;
-    k_collect_leaves<<<grid_for(C.cap, 256, 4 * c->num_sms), 256, 0, c->stream>>>(
-        C.nchild, C.first, C.count, c->ctl, C.cap, C.leaves, &c->ctl->n_leaves, C.leaf_of, gate);
-    c->launches++;
-    NCORP_CUDA_CHECK(cudaGetLastError());
 }
 
 // ---------------------------------------------------------------------------
@@ -944,7 +907,7 @@ void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double 
     // every SM: the FP64 work of the leaves and of theta(M) is bound by the FP64 units of the
     // sub-partitions, so it is spread over all of them
     const int grid = coop_grid(c, reinterpret_cast<const void *>(k_geometry), block, 0);
-    void *args[] = {&A};   // ctl->bar_count was zeroed by k_collect_leaves
+    void *args[] = {&A};   // ctl->bar_count was zeroed by k_build
     NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_geometry), dim3(grid), dim3(block),
                                                  args, 0, c->stream));
     c->launches++;
