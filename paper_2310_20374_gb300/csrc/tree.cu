@@ -313,8 +313,33 @@ void launch_build(ncorp_ctx *c, const ParticleSet &P, int n, int s, const int *g
 // Corner cap (Sect. 3.4.2): distance from s to the farthest corner of the
 // cell's cube, the cube widened by L 2^-48 on each side.
 // ---------------------------------------------------------------------------
+// One FP64 warp instruction takes 64 cycles of its SM sub-partition, a divide
+// 550, a square root 584, a compare and select 111, a conversion 84.  So what
+// only looks at an FP64 value's bits is done in integers: maxima and compares
+// of values that are not negative, scalings by powers of two.
+
+// v 2^e for a power of two v (or 0): exact, as ldexp
+__device__ __forceinline__ double scale_pow2(double v, int e) {
+    const long long u = __double_as_longlong(v);
+    const int ex = static_cast<int>(u >> 52) & 0x7ff;
+    if (ex + e > 0 && ex + e < 0x7ff && ex > 0) return __longlong_as_double(u + (static_cast<long long>(e) << 52));
+    return ldexp(v, e);
+}
+
+// the larger of a >= 0 and b, b taken as 0 when it is NaN or negative (fmax of a >= 0 and b)
+__device__ __forceinline__ double max_nn(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return (y > x && y <= 0x7ff0000000000000ll) ? b : a;
+}
+
+// a < b for values that are not negative (false when b is NaN or a is)
+__device__ __forceinline__ bool less_nn(double a, double b) {
+    const long long x = __double_as_longlong(a), y = __double_as_longlong(b);
+    return x < y && y <= 0x7ff0000000000000ll;
+}
+
 // root: the cube of the cell's disk (x_lo, y_lo, z_lo, L)
-__device__ __forceinline__ double cell_side(const double *root, int lev) { return ldexp(root[3], -lev); }
+__device__ __forceinline__ double cell_side(const double *root, int lev) { return scale_pow2(root[3], -lev); }
 
 // the root cube of cell c's disk
 __device__ __forceinline__ const double *cell_root(const Ctrl *ctl, const int *first, int c) {
@@ -322,34 +347,40 @@ __device__ __forceinline__ const double *cell_root(const Ctrl *ctl, const int *f
 }
 
 __device__ __forceinline__ double corner_axis(const double *root, int k, double h, uint32_t c, double s) {
-    const double eps = dmul(root[3], 0x1p-48);
-    const double lo = dadd(root[k], dmul(static_cast<double>(c), h));
+    const double eps = scale_pow2(root[3], -48);
+    const double lo = dadd(root[k], dmul(__dsub_rn(__hiloint2double(0x43300000, static_cast<int>(c)), 0x1p52), h));
     const double a = dsub(s, dsub(lo, eps));
     const double b = dsub(dadd(dadd(lo, h), eps), s);
-    return a > b ? a : b;
+    // (a + b = h + 2 eps > 0: at most one is negative, so the integer order is the values')
+    return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
 }
 
-__device__ __forceinline__ double corner_distance(const double *root, int lev, uint32_t cx, uint32_t cy, uint32_t cz,
-                                                  double sx, double sy, double sz) {
-    const double h = cell_side(root, lev);
-    return dnorm3(corner_axis(root, 0, h, cx, sx), corner_axis(root, 1, h, cy, sy), corner_axis(root, 2, h, cz, sz));
-}
-
-// Power-of-two scale of a cell's expansions: >= r_max (so |x - s|/rho <= 1)
+// Power-of-two scale of a cell's expansions: the smallest >= r_max (so |x - s|/rho <= 1)
 // and >= side/256, so that the scale ratios met in M2M, M2L and L2L stay
 // below 2^(level difference + 8) even for one-moonlet cells (r_max ~ 0).
 __device__ __forceinline__ double cell_scale(const double *root, int lev, double rmax) {
-    return pow2_ceil(fmax(rmax, cell_side(root, lev) * 0x1p-8));
+    const double v = max_nn(rmax, scale_pow2(cell_side(root, lev), -8));
+    const long long u = __double_as_longlong(v);
+    const int ex = static_cast<int>(u >> 52) & 0x7ff;
+    if (ex == 0 || ex >= 0x7fe) return pow2_ceil(v);
+    return __longlong_as_double((u & 0xfffffffffffffll) ? static_cast<long long>(ex + 1) << 52 : u);
 }
 
-// FP32 double-float copy of a centre: hi = fl32(s), lo = fl32(s - hi)
-__device__ __forceinline__ void split3(double x, double y, double z, float4 &hi, float4 &lo) {
-    hi.x = static_cast<float>(x);
-    hi.y = static_cast<float>(y);
-    hi.z = static_cast<float>(z);
-    lo.x = static_cast<float>(x - static_cast<double>(hi.x));
-    lo.y = static_cast<float>(y - static_cast<double>(hi.y));
-    lo.z = static_cast<float>(z - static_cast<double>(hi.z));
+// FP32 double-float copy of a coordinate: hi = fl32(v), lo = fl32(v - hi)
+__device__ __forceinline__ void split1(double v, float &hi, float &lo) {
+    hi = static_cast<float>(v);
+    lo = static_cast<float>(v - static_cast<double>(hi));
+}
+
+// The three coordinates of a centre, one on each of lanes base + first .. + 2, as FP32 pairs on every lane
+__device__ __forceinline__ void gather_split(float h, float l, int from, float4 &hi, float4 &lo) {
+    hi.x = __shfl_sync(0xffffffffu, h, from);
+    hi.y = __shfl_sync(0xffffffffu, h, from + 1);
+    hi.z = __shfl_sync(0xffffffffu, h, from + 2);
+    lo.x = __shfl_sync(0xffffffffu, l, from);
+    lo.y = __shfl_sync(0xffffffffu, l, from + 1);
+    lo.z = __shfl_sync(0xffffffffu, l, from + 2);
+    hi.w = lo.w = 0.f;
 }
 
 // ---------------------------------------------------------------------------
@@ -373,6 +404,7 @@ struct ClimbArgs {
     const int *leaves;
     Ctrl *ctl;
     double G, dt, theta;
+    double K3;                // (theta_min^5 / (1 - theta_min)^2)^3
     int cap;
     const double *rc_given;   // collision climb (nullable): each moonlet's R + dt |v| given (tree order)
     const int *gate;          // collision climb (nullable): nothing to do while *gate is 0
@@ -412,15 +444,48 @@ __device__ __forceinline__ LeafSlot leaf_slot(const ClimbArgs &A, int gw, int la
     return L;
 }
 
-__device__ __forceinline__ double quad_max(double v) {
-    v = fmax(v, __shfl_xor_sync(0xffffffffu, v, 1));
-    return fmax(v, __shfl_xor_sync(0xffffffffu, v, 2));
+__device__ __forceinline__ double quad_max(double v) {   // (of values that are not negative)
+    v = max_nn(v, __shfl_xor_sync(0xffffffffu, v, 1));
+    return max_nn(v, __shfl_xor_sync(0xffffffffu, v, 2));
 }
+
+// The largest of a leaf's values, found in FP32: every lane keeps the largest
+// and second largest FP32 estimate of its quarter and where the largest is.
+// After the quad's maximum is known, only the moonlets whose estimate reaches
+// it within the estimates' error (2^-18 of it, four times the bound) need the
+// exact FP64 value: one a leaf as a rule, evaluated once for the whole warp.
+// A leaf whose estimates may not show it (a second candidate on one lane, values
+// that are not finite or too small to carry their relative error) is left to
+// the exact loop over its moonlets: settle() is false on its four lanes.
+struct LeafMax {
+    float best = -1.f, second = -1.f;
+    int at = -1;
+    bool odd = false;      // an estimate that says nothing
+    __device__ __forceinline__ void add(float v, int k) {
+        if (!(v >= 0.f && v < 3e38f)) odd = true;
+        if (v > best) {
+            second = best;
+            best = v;
+            at = k;
+        } else if (v > second) {
+            second = v;
+        }
+    }
+    // floor_: values at or below it say nothing.  On true, `at` is the lane's candidate (-1: none).
+    __device__ __forceinline__ bool settle(float floor_, int base) {
+        float m = fmaxf(best, __shfl_xor_sync(0xffffffffu, best, 1));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+        const float thr = m * (1.0f - 0x1p-18f);
+        const bool ok = !odd && m > floor_ && !(second >= thr);
+        if (!(best >= thr)) at = -1;
+        return ((__ballot_sync(0xffffffffu, ok) >> base) & 0xfu) == 0xfu;
+    }
+};
 
 // Corner cap of the leaf (lanes q = 0..2 take one axis each), returned on every lane of the quad.
 __device__ __forceinline__ double quad_corner(const ClimbArgs &A, const LeafSlot &L, double sx, double sy, double sz) {
     double d = 0.0;
-    if (L.valid && L.q < 3) {
+    if (L.valid && L.q < 3) {   // (lanes of the other quads run with it)
         const int lev = A.level[L.c];
         const double *rt = disk_root(A.ctl, disk_of(A.ctl, L.f));
         const double h = cell_side(rt, lev);
@@ -432,27 +497,53 @@ __device__ __forceinline__ double quad_corner(const ClimbArgs &A, const LeafSlot
     return dnorm3(d0, d1, d2);
 }
 
+// FP32 estimate of |x_k - s|^2 of moonlet k, s given as FP32 pairs
+__device__ __forceinline__ float dist2_f32(const float4 &h, const float4 &l, const float4 &sh, const float4 &sl) {
+    const float dx = (h.x - sh.x) + (l.x - sl.x), dy = (h.y - sh.y) + (l.y - sl.y), dz = (h.z - sh.z) + (l.z - sl.z);
+    return dx * dx + dy * dy + dz * dz;
+}
+
+// max_k |x_k - s|^2 of the quad's leaf, exact, on every lane of the quad; sh, sl: the centre in FP32 pairs
+// (which carry an absolute error of 2^-47 |s|: distances below 2^-20 |s| are left to the exact loop)
+__device__ __forceinline__ double leaf_dist2(const ClimbArgs &A, const LeafSlot &L, double sx, double sy, double sz,
+                                             const float4 &sh, const float4 &sl) {
+    LeafMax M;
+    for (int k = L.f + L.q; k < L.f + L.cnt; k += 4) M.add(dist2_f32(A.hi4[k], A.lo4[k], sh, sl), k);
+    const float fl = (fabsf(sh.x) + fabsf(sh.y) + fabsf(sh.z)) * 0x1p-20f;
+    double d2 = 0.0;
+    if (M.settle(fl * fl + 1e-30f, L.base)) {
+        const int k = M.at;
+        if (k >= 0) d2 = dsq3(dsub(A.x[k], sx), dsub(A.y[k], sy), dsub(A.z[k], sz));
+    } else {
+        for (int k = L.f + L.q; k < L.f + L.cnt; k += 4)
+            d2 = max_nn(d2, dsq3(dsub(A.x[k], sx), dsub(A.y[k], sy), dsub(A.z[k], sz)));
+    }
+    __syncwarp();
+    return quad_max(max_nn(0.0, d2));
+}
+
 // ---- gravity leaves (Eqs. expansion_center, rmax_2, corner cap): the
 // group of LEAF_GROUP leaves of warp-group gw.
 __device__ __forceinline__ void leaf_gravity_group(const ClimbArgs &A, int gw, int lane, int n_leaves) {
     const LeafSlot L = leaf_slot(A, gw, lane, n_leaves);
     const double *coord = L.q == 1 ? A.x : (L.q == 2 ? A.y : A.z);
     double acc = 0.0;
+#pragma unroll 4
     for (int k = L.f; k < L.f + L.cnt; k++) {
-        const double m = A.m[k];
-        acc = L.q == 0 ? dadd(acc, m) : dadd(acc, dmul(m, coord[k]));
+        const double m = A.m[k], c = coord[k];
+        acc = dadd(acc, L.q == 0 ? m : dmul(m, c));
     }
     const double M = __shfl_sync(0xffffffffu, acc, L.base);
     const double sq = L.q == 0 ? M : ddiv(acc, M);
     const double sx = __shfl_sync(0xffffffffu, sq, L.base + 1), sy = __shfl_sync(0xffffffffu, sq, L.base + 2),
                  sz = __shfl_sync(0xffffffffu, sq, L.base + 3);
-    double d2 = 0.0;
-    for (int k = L.f + L.q; k < L.f + L.cnt; k += 4)
-        d2 = fmax(d2, dsq3(dsub(A.x[k], sx), dsub(A.y[k], sy), dsub(A.z[k], sz)));
-    d2 = quad_max(d2);
-    double rmax = dsqrt(d2);
+    float h1, l1;
+    split1(sq, h1, l1);
+    float4 hi, lo;
+    gather_split(h1, l1, L.base + 1, hi, lo);
+    double rmax = dsqrt(leaf_dist2(A, L, sx, sy, sz, hi, lo));
     const double cap = quad_corner(A, L, sx, sy, sz);
-    if (cap < rmax) rmax = cap;
+    if (less_nn(cap, rmax)) rmax = cap;
     if (L.valid && L.q == 0) {
         const int c = L.c;
         const double rho = cell_scale(cell_root(A.ctl, A.first, c), A.level[c], rmax);
@@ -462,9 +553,6 @@ __device__ __forceinline__ void leaf_gravity_group(const ClimbArgs &A, int gw, i
         A.sz[c] = sz;
         A.rmax[c] = rmax;
         A.rho[c] = rho;
-        float4 hi, lo;
-        split3(sx, sy, sz, hi, lo);
-        hi.w = 0.f;
         lo.w = static_cast<float>(rho);
         A.gh[c] = hi;
         A.gl[c] = lo;
@@ -510,6 +598,22 @@ __device__ __forceinline__ void store_reduced(real *acc, real *dst, int lane) {
 // the group's parent, -1 for none; every lane of the warp calls this.
 constexpr int PARENT_GROUP = 4;
 
+// Sums over a parent's children in child order: lane 0 of its eight the
+// weights w, lanes 1..3 the weighted coordinates; lane j < nch gives child j's.
+// Each lane forms its own child's products, so a child costs the sums one FP64
+// addition.
+__device__ __forceinline__ double children_sum(double w, double x, double y, double z, int nch, int j, int base) {
+    const double wx = dmul(w, x), wy = dmul(w, y), wz = dmul(w, z);
+    const int most = __reduce_max_sync(0xffffffffu, nch);
+    double acc = 0.0;
+    for (int ch = 0; ch < most; ch++) {
+        const double a = __shfl_sync(0xffffffffu, w, base + ch), bx = __shfl_sync(0xffffffffu, wx, base + ch),
+                     by = __shfl_sync(0xffffffffu, wy, base + ch), bz = __shfl_sync(0xffffffffu, wz, base + ch);
+        if (ch < nch) acc = dadd(acc, j == 1 ? bx : (j == 2 ? by : (j == 3 ? bz : a)));
+    }
+    return acc;
+}
+
 __device__ __forceinline__ void parent_gravity_group(const ClimbArgs &A, int c, int lane) {
     const int j = lane & 7, base = lane & ~7;
     const bool valid = c >= 0;
@@ -522,26 +626,20 @@ __device__ __forceinline__ void parent_gravity_group(const ClimbArgs &A, int c, 
         csz = __ldcg(&A.sz[c0 + j]);
         crm = __ldcg(&A.rmax[c0 + j]);
     }
-    double acc = 0.0;
-#pragma unroll
-    for (int ch = 0; ch < 8; ch++) {
-        const double w = __shfl_sync(0xffffffffu, cm, base + ch);
-        const double bx = __shfl_sync(0xffffffffu, csx, base + ch);
-        const double by = __shfl_sync(0xffffffffu, csy, base + ch);
-        const double bz = __shfl_sync(0xffffffffu, csz, base + ch);
-        const double coord = j == 1 ? bx : (j == 2 ? by : (j == 3 ? bz : 1.0));
-        const double t = dmul(w, coord);
-        if (ch < nch) acc = dadd(acc, t);
-    }
+    const double acc = children_sum(cm, csx, csy, csz, nch, j, base);
     const double M = __shfl_sync(0xffffffffu, acc, base);
     const double q = ddiv(acc, M);
     const double px = __shfl_sync(0xffffffffu, q, base + 1), py = __shfl_sync(0xffffffffu, q, base + 2),
                  pz = __shfl_sync(0xffffffffu, q, base + 3);
     double rm = 0.0;
     if (j < nch) rm = dadd(crm, dnorm3(dsub(csx, px), dsub(csy, py), dsub(csz, pz)));
-    rm = fmax(rm, __shfl_xor_sync(0xffffffffu, rm, 1));
-    rm = fmax(rm, __shfl_xor_sync(0xffffffffu, rm, 2));
-    rm = fmax(rm, __shfl_xor_sync(0xffffffffu, rm, 4));
+    rm = max_nn(0.0, rm);
+#pragma unroll
+    for (int o = 1; o < 8; o <<= 1) rm = max_nn(rm, __shfl_xor_sync(0xffffffffu, rm, o));
+    float h1, l1;
+    split1(q, h1, l1);
+    float4 hi, lo;
+    gather_split(h1, l1, base + 1, hi, lo);
     const int plev = valid ? A.level[c] : 0;
     double d = 0.0;
     if (valid && j < 3) {
@@ -552,7 +650,7 @@ __device__ __forceinline__ void parent_gravity_group(const ClimbArgs &A, int c, 
     const double d0 = __shfl_sync(0xffffffffu, d, base), d1 = __shfl_sync(0xffffffffu, d, base + 1),
                  d2 = __shfl_sync(0xffffffffu, d, base + 2);
     const double pcap = dnorm3(d0, d1, d2);
-    if (pcap < rm) rm = pcap;
+    if (less_nn(pcap, rm)) rm = pcap;
     if (valid && j == 0) {
         const double prho = cell_scale(cell_root(A.ctl, A.first, c), plev, rm);
         A.M[c] = M;
@@ -561,9 +659,6 @@ __device__ __forceinline__ void parent_gravity_group(const ClimbArgs &A, int c, 
         A.sz[c] = pz;
         A.rmax[c] = rm;
         A.rho[c] = prho;
-        float4 hi, lo;
-        split3(px, py, pz, hi, lo);
-        hi.w = 0.f;
         lo.w = static_cast<float>(prho);
         A.gh[c] = hi;
         A.gl[c] = lo;
@@ -822,33 +917,51 @@ static void p2m_t(ncorp_ctx *c, const P2MArgs &B) {
 // K = theta_min^5/(1-theta_min)^2, i.e. the root in [theta_min, 1) of the
 // increasing f(theta) = theta^15 M - K^3 M_tot (1-theta)^6: 12 bisection
 // steps, then 4 Newton steps kept inside the final bracket (+ - x / only).
-__device__ double theta_of(double M, double Mtot, double tmin) {
-    const double t2 = dmul(tmin, tmin), t4 = dmul(t2, t2), t5 = dmul(t4, tmin);
-    const double u = dsub(1.0, tmin), u2 = dmul(u, u);
-    const double K = ddiv(t5, u2);
-    const double K3 = dmul(dmul(K, K), K);
-    const double rhs = dmul(K3, Mtot);
+// K3 = K^3, rhs = K^3 M_tot in FP64; tmin > 0.
+// A bisection step only needs the sign of f, so it is taken from FP32 values
+// of the two terms when they differ by more than their error (theta and its
+// complement cut to FP32: 2^-23 each, 15 and 6 powers, the roundings of the
+// products: below 2^-18 + 2^-20 / (1 - theta) together), else from FP64: one
+// FP64 instruction a step in place of fourteen.
+__device__ double theta_of(double M, double rhs, double tmin) {
     double lo = tmin, hi = 1.0;
+    const float Mf = static_cast<float>(M), rf = static_cast<float>(rhs);
+    const bool small = !(Mf > 1e-15f && Mf < 1e15f && rf > 1e-15f && rf < 1e15f);   // (products may leave the FP32 range)
+#pragma unroll 1
     for (int it = 0; it < 12; it++) {
-        const double mid = dmul(dadd(lo, hi), 0.5);
-        const double m2 = dmul(mid, mid), m3 = dmul(m2, mid), m6 = dmul(m3, m3), m12 = dmul(m6, m6),
-                     m15 = dmul(m12, m3);
-        const double w = dsub(1.0, mid), w2 = dmul(w, w), w3 = dmul(w2, w), w6 = dmul(w3, w3);
-        const double f = dsub(dmul(m15, M), dmul(rhs, w6));
-        if (f > 0.0) hi = mid;
+        const double sum = dadd(lo, hi);   // in (0, 2): halved exactly by its exponent
+        const double mid = __longlong_as_double(__double_as_longlong(sum) - (1ll << 52));
+        // mid in FP32 (cut): 0 < mid < 1
+        const unsigned mh = static_cast<unsigned>(__double2hiint(mid)), ml = static_cast<unsigned>(__double2loint(mid));
+        const float t = (mh >> 20) > 900u ? __uint_as_float(((mh - (896u << 20)) << 3) | (ml >> 29)) : 0.f;
+        const float w = 1.0f - t;
+        const float t2 = t * t, t3 = t2 * t, t6 = t3 * t3, t12 = t6 * t6, w2 = w * w, w4 = w2 * w2;
+        const float a = t12 * t3 * Mf, c = w4 * w2 * rf;
+        const float margin = (0x1p-17f + 0x1p-19f / w) * fmaxf(a, c);
+        bool up;   // f > 0
+        if (small || !(t12 > 1e-15f && w4 > 1e-12f) || !(fabsf(a - c) > margin)) {
+            const double m2 = dmul(mid, mid), m3 = dmul(m2, mid), m6 = dmul(m3, m3), m12 = dmul(m6, m6),
+                         m15 = dmul(m12, m3);
+            const double v = dsub(1.0, mid), v2 = dmul(v, v), v3 = dmul(v2, v), v6 = dmul(v3, v3);
+            up = dsub(dmul(m15, M), dmul(rhs, v6)) > 0.0;
+        } else {
+            up = a > c;
+        }
+        if (up) hi = mid;
         else lo = mid;
     }
     double th = dmul(dadd(lo, hi), 0.5);
+    const double rhs6 = dmul(6.0, rhs);
     for (int it = 0; it < 4; it++) {
         const double w = dsub(1.0, th);
         const double q2 = dmul(th, th), q3 = dmul(q2, th), q6 = dmul(q3, q3), q12 = dmul(q6, q6),
                      q14 = dmul(q12, q2), q15 = dmul(q14, th);
         const double w2 = dmul(w, w), w3 = dmul(w2, w), w5 = dmul(w3, w2), w6 = dmul(w3, w3);
         const double f = dsub(dmul(q15, M), dmul(rhs, w6));
-        const double fp = dadd(dmul(dmul(15.0, q14), M), dmul(dmul(6.0, rhs), w5));
+        const double fp = dadd(dmul(dmul(15.0, q14), M), dmul(rhs6, w5));
         double nt = dsub(th, ddiv(f, fp));
-        if (nt < lo) nt = lo;
-        if (nt > hi) nt = hi;
+        if (__double_as_longlong(nt) < __double_as_longlong(lo)) nt = lo;   // (lo > 0: a negative nt too)
+        if (less_nn(hi, nt)) nt = hi;
         th = nt;
     }
     return th;
@@ -886,7 +999,7 @@ __global__ void __launch_bounds__(32 * CLIMB_WARPS_COOP) k_geometry(ClimbArgs A)
     {
         for (int i = gw0 * 32 + lane; i < nc; i += nwarps * 32) {
             const double Mtot = __ldcg(&A.M[disk_of(A.ctl, A.first[i])]);
-            const double rc = ddiv(__ldcg(&A.rmax[i]), theta_of(__ldcg(&A.M[i]), Mtot, A.theta));
+            const double rc = ddiv(__ldcg(&A.rmax[i]), theta_of(__ldcg(&A.M[i]), dmul(A.K3, Mtot), A.theta));
             A.rcrit[i] = rc;
             A.gh[i].w = static_cast<float>(rc);
         }
@@ -903,6 +1016,11 @@ void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double 
     A.M = C.M; A.sx = C.sx; A.sy = C.sy; A.sz = C.sz; A.rmax = C.rmax; A.rcrit = C.rcrit; A.rho = C.rho;
     A.gh = C.gh; A.gl = C.gl;
     A.Mh = C.Mh; A.leaves = C.leaves; A.ctl = c->ctl; A.G = G; A.theta = theta; A.cap = C.cap;
+    {   // K^3, each operation rounded once as on the device (no contraction: products and quotients only)
+        const double t2 = theta * theta, t4 = t2 * t2, t5 = t4 * theta, u = 1.0 - theta, u2 = u * u, K = t5 / u2;
+        const double K2 = K * K;
+        A.K3 = K2 * K;
+    }
     const int block = 32 * CLIMB_WARPS_COOP;
     // every SM: the FP64 work of the leaves and of theta(M) is bound by the FP64 units of the
     // sub-partitions, so it is spread over all of them
@@ -940,11 +1058,21 @@ void launch_multipoles(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, do
     NCORP_CUDA_CHECK(cudaGetLastError());
 }
 
+// FP64 value cut to FP32 in integers (relative error below 2^-23; beyond the FP32 range: 0, infinity; NaN stays NaN)
+__device__ __forceinline__ float cut_f32(double v) {
+    const unsigned h = static_cast<unsigned>(__double2hiint(v)), l = static_cast<unsigned>(__double2loint(v));
+    const int ex = static_cast<int>((h >> 20) & 0x7ff) - 896;
+    const unsigned sign = h & 0x80000000u;
+    if (ex <= 0) return __uint_as_float(sign);
+    if (ex >= 255) return (ex == 0x7ff - 896 && ((h & 0xfffffu) | l)) ? __uint_as_float(0x7fffffffu) : __uint_as_float(sign | 0x7f800000u);
+    return __uint_as_float(sign | (static_cast<unsigned>(ex) << 23) | ((h & 0xfffffu) << 3) | (l >> 29));
+}
+
 // ---------------------------------------------------------------------------
 // Collision climb (Eqs. center, rmax, rcrit): s-bar is the mean moonlet
 // position (children weighted by their moonlet counts); r_crit = r_max + max
 // over children of (r_crit - r_max), a moonlet's being R + dt |v| (stored,
-// rounded up to FP32, with the velocity rounded to FP32, for the pair
+// as an FP32 upper bound, with the velocity in FP32, for the pair
 // prefilter).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(64) k_leaf_collision(ClimbArgs A) {
@@ -955,33 +1083,56 @@ __global__ void __launch_bounds__(64) k_leaf_collision(ClimbArgs A) {
     const int lane = threadIdx.x & 31;
     const int n_leaves = A.ctl->n_leaves;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const float dtf = static_cast<float>(A.dt);
     for (int gw = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; gw * LEAF_GROUP < n_leaves; gw += nwarps) {
         const LeafSlot L = leaf_slot(A, gw, lane, n_leaves);
         const double *coord = L.q == 0 ? A.x : (L.q == 1 ? A.y : A.z);
         double acc = 0.0;
-        if (L.q < 3)
-            for (int k = L.f; k < L.f + L.cnt; k++) acc = dadd(acc, coord[k]);
-        const double sq = L.q < 3 ? ddiv(acc, static_cast<double>(L.cnt)) : 0.0;
+#pragma unroll 4
+        for (int k = L.f; k < L.f + L.cnt; k++) acc = dadd(acc, coord[k]);
+        const double sq = ddiv(acc, static_cast<double>(L.valid ? L.cnt : 1));
         const double sx = __shfl_sync(0xffffffffu, sq, L.base), sy = __shfl_sync(0xffffffffu, sq, L.base + 1),
                      sz = __shfl_sync(0xffffffffu, sq, L.base + 2);
-        double d2 = 0.0, ex = 0.0;
-        for (int k = L.f + L.q; k < L.f + L.cnt; k += 4) {
-            d2 = fmax(d2, dsq3(dsub(A.x[k], sx), dsub(A.y[k], sy), dsub(A.z[k], sz)));
-            if (A.rc_given) {   // bounds given: the pair test's per-moonlet values come later
-                ex = fmax(ex, A.rc_given[k]);
-                continue;
+        float h1, l1;
+        split1(sq, h1, l1);
+        float4 hi, lo;
+        gather_split(h1, l1, L.base, hi, lo);
+        const double d2 = leaf_dist2(A, L, sx, sy, sz, hi, lo);
+        // the largest R + dt |v|: estimated in FP32 like the distances; the estimate's upper bound goes to the
+        // pair test, which needs R + dt |v| from above
+        double ex = 0.0;
+        if (A.rc_given) {   // bounds given: the pair test's per-moonlet values come later
+            for (int k = L.f + L.q; k < L.f + L.cnt; k += 4) ex = max_nn(ex, A.rc_given[k]);
+        } else {
+            LeafMax E;
+            for (int k = L.f + L.q; k < L.f + L.cnt; k += 4) {
+                const float vx = cut_f32(A.vx[k]), vy = cut_f32(A.vy[k]), vz = cut_f32(A.vz[k]), r = cut_f32(A.R[k]);
+                const float v2 = vx * vx + vy * vy + vz * vz;
+                float e, up;
+                if (r >= 0.f && v2 > 1e-30f && v2 < 1e30f) {
+                    e = r + dtf * sqrtf(v2);
+                    up = e * (1.0f + 0x1p-19f);
+                } else {   // at rest, a negative radius, or speeds whose squares leave the FP32 range
+                    const double x = dadd(A.R[k], dmul(A.dt, dnorm3(A.vx[k], A.vy[k], A.vz[k])));
+                    e = static_cast<float>(x);
+                    up = __double2float_ru(x);
+                }
+                E.add(e, k);
+                A.cv4[k] = make_float4(vx, vy, vz, up);
             }
-            const double vx = A.vx[k], vy = A.vy[k], vz = A.vz[k];
-            const double e = dadd(A.R[k], dmul(A.dt, dnorm3(vx, vy, vz)));
-            ex = fmax(ex, e);
-            A.cv4[k] = make_float4(static_cast<float>(vx), static_cast<float>(vy), static_cast<float>(vz),
-                                   __double2float_ru(e));
+            if (E.settle(1e-35f, L.base)) {
+                const int k = E.at;
+                if (k >= 0) ex = dadd(A.R[k], dmul(A.dt, dnorm3(A.vx[k], A.vy[k], A.vz[k])));
+            } else {
+                for (int k = L.f + L.q; k < L.f + L.cnt; k += 4)
+                    ex = max_nn(ex, dadd(A.R[k], dmul(A.dt, dnorm3(A.vx[k], A.vy[k], A.vz[k]))));
+            }
+            __syncwarp();
         }
-        d2 = quad_max(d2);
-        ex = quad_max(ex);
+        ex = quad_max(max_nn(0.0, ex));
         double rmax = dsqrt(d2);
         const double cap = quad_corner(A, L, sx, sy, sz);
-        if (cap < rmax) rmax = cap;
+        if (less_nn(cap, rmax)) rmax = cap;
         if (L.valid && L.q == 0) {
             const int c = L.c;
             const double rc = dadd(rmax, ex);
@@ -990,10 +1141,7 @@ __global__ void __launch_bounds__(64) k_leaf_collision(ClimbArgs A) {
             A.sz[c] = sz;
             A.rmax[c] = rmax;
             A.rcrit[c] = rc;
-            float4 hi, lo;
-            split3(sx, sy, sz, hi, lo);
             hi.w = static_cast<float>(rc);
-            lo.w = 0.f;
             A.gh[c] = hi;
             A.gl[c] = lo;
         }
@@ -1019,27 +1167,23 @@ __device__ __forceinline__ void parent_collision_group(const ClimbArgs &A, int c
         crm = __ldcg(&A.rmax[c0 + j]);
         cex = dsub(__ldcg(&A.rcrit[c0 + j]), crm);
     }
-    double acc = 0.0;
-#pragma unroll
-    for (int ch = 0; ch < 8; ch++) {
-        const double w = __shfl_sync(0xffffffffu, cw, base + ch);
-        const double bx = __shfl_sync(0xffffffffu, csx, base + ch);
-        const double by = __shfl_sync(0xffffffffu, csy, base + ch);
-        const double bz = __shfl_sync(0xffffffffu, csz, base + ch);
-        const double coord = j == 1 ? bx : (j == 2 ? by : (j == 3 ? bz : 1.0));
-        const double t = dmul(w, coord);
-        if (ch < nch) acc = dadd(acc, t);
-    }
+    const double acc = children_sum(cw, csx, csy, csz, nch, j, base);
     const double q = ddiv(acc, valid ? static_cast<double>(A.count[c]) : 1.0);
     const double px = __shfl_sync(0xffffffffu, q, base + 1), py = __shfl_sync(0xffffffffu, q, base + 2),
                  pz = __shfl_sync(0xffffffffu, q, base + 3);
     double rm = 0.0;
     if (j < nch) rm = dadd(crm, dnorm3(dsub(csx, px), dsub(csy, py), dsub(csz, pz)));
+    rm = max_nn(0.0, rm);
+    cex = max_nn(0.0, cex);
 #pragma unroll
     for (int o = 1; o < 8; o <<= 1) {
-        rm = fmax(rm, __shfl_xor_sync(0xffffffffu, rm, o));
-        cex = fmax(cex, __shfl_xor_sync(0xffffffffu, cex, o));
+        rm = max_nn(rm, __shfl_xor_sync(0xffffffffu, rm, o));
+        cex = max_nn(cex, __shfl_xor_sync(0xffffffffu, cex, o));
     }
+    float h1, l1;
+    split1(q, h1, l1);
+    float4 hi, lo;
+    gather_split(h1, l1, base + 1, hi, lo);
     double d = 0.0;
     if (valid && j < 3) {
         const double *rt = cell_root(A.ctl, A.first, c);
@@ -1049,7 +1193,7 @@ __device__ __forceinline__ void parent_collision_group(const ClimbArgs &A, int c
     const double d0 = __shfl_sync(0xffffffffu, d, base), d1 = __shfl_sync(0xffffffffu, d, base + 1),
                  d2 = __shfl_sync(0xffffffffu, d, base + 2);
     const double pcap = dnorm3(d0, d1, d2);
-    if (pcap < rm) rm = pcap;
+    if (less_nn(pcap, rm)) rm = pcap;
     if (valid && j == 0) {
         const double rc = dadd(rm, cex);
         A.sx[c] = px;
@@ -1057,10 +1201,7 @@ __device__ __forceinline__ void parent_collision_group(const ClimbArgs &A, int c
         A.sz[c] = pz;
         A.rmax[c] = rm;
         A.rcrit[c] = rc;
-        float4 hi, lo;
-        split3(px, py, pz, hi, lo);
         hi.w = static_cast<float>(rc);
-        lo.w = 0.f;
         A.gh[c] = hi;
         A.gl[c] = lo;
     }
@@ -1093,6 +1234,7 @@ void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx
     Cells &C = c->cells;
     ClimbArgs A{};
     A.x = P.x; A.y = P.y; A.z = P.z; A.R = P.R; A.vx = vx; A.vy = vy; A.vz = vz;
+    A.hi4 = P.hi4; A.lo4 = P.lo4;
     A.first = C.first; A.count = C.count; A.child0 = C.child0; A.nchild = C.nchild; A.parent = C.parent;
     A.level = C.level; A.arrive = C.arrive; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
     A.sx = C.bx; A.sy = C.by; A.sz = C.bz; A.rmax = C.bmax; A.rcrit = C.bcrit;
