@@ -562,13 +562,15 @@ int finish(ncorp_ctx *c, bool both = false) {
 // gate (nullable, radix sort only): every kernel does nothing while *gate is 0.
 // spec_dt > 0 (fused walk): the gather also bounds every moonlet's next R + dt |v| (velocities of sv,
 // accelerations of sr)
+// keyed: called once the keys are enqueued, before their sort
+template <class F>
 void build_tree(ncorp_ctx *c, const ParticleSet &sx, const ParticleSet &sv, const ParticleSet &sr, ParticleSet &dst,
-                int n, bool near_sorted = false, bool bbox_done = false, const int *gate = nullptr,
-                double spec_dt = 0.0) {
+                int n, bool near_sorted, bool bbox_done, const int *gate, double spec_dt, F keyed) {
     c->cur_n = n;
     {
         Stage st(c, NCORP_STAGE_SORT);
         launch_bbox_keys(c, sx.x, sx.y, sx.z, n, dst.key, c->B.qx, c->B.qy, c->B.qz, bbox_done, gate);
+        keyed();
         // (a forest's keys restart in every disk: they are sorted by (disk, key) with the full radix sort)
         if (near_sorted && c->nd == 1) sort_near_sorted(c, dst.key, c->idx, c->key_alt, c->idx_alt, n, 3 * KEY_BITS);
         else radix_sort_u64(c, dst.key, c->idx, c->key_alt, c->idx_alt, n, 3 * KEY_BITS, true, gate, true);
@@ -580,6 +582,12 @@ void build_tree(ncorp_ctx *c, const ParticleSet &sx, const ParticleSet &sv, cons
     }
     Stage st(c, NCORP_STAGE_BUILD);
     launch_build(c, dst, n, c->s, gate);
+}
+
+void build_tree(ncorp_ctx *c, const ParticleSet &sx, const ParticleSet &sv, const ParticleSet &sr, ParticleSet &dst,
+                int n, bool near_sorted = false, bool bbox_done = false, const int *gate = nullptr,
+                double spec_dt = 0.0) {
+    build_tree(c, sx, sv, sr, dst, n, near_sorted, bbox_done, gate, spec_dt, [] {});
 }
 
 // Runs body with c->stream set to s (launchers enqueue on c->stream).
@@ -733,8 +741,9 @@ void enqueue_kdk(ncorp_ctx *c, int n, int p, double theta, double dt, bool overl
         K.cv4 = c->cv4;
         launch_kick_drift(c, K);
     }
-    if (c->cfg.collisions) {
-        if (side) {
+    // the search on the side stream, beside what the main stream does next; called with A's tree set as the other one
+    auto fork_search = [&] {
+        on_alt(c, [&] {
             cudaStream_t main = c->stream;
             const int cap = c->coop_max;
             NCORP_CUDA_CHECK(cudaEventRecord(c->ev_fork, main));
@@ -752,18 +761,26 @@ void enqueue_kdk(ncorp_ctx *c, int n, int p, double theta, double dt, bool overl
             }
             c->stream = main;
             c->coop_max = cap;
-        } else {
-            collisions(c, A, B.vx, B.vy, B.vz, dt, false);   // (no overlap: a batch's streams share the GPU)
-            if (resolve) {
-                Stage st(c, NCORP_STAGE_COLLIDE);
-                launch_resolve(c, A, B, n, dt);
-                // the drifted box again, if a moonlet's drift changed (the new tree set's control block)
-                launch_bbox_gated(c, B.x, B.y, B.z, n, c->alt.ctl, &c->ctl->n_resolved);
-            }
+        });
+    };
+    if (c->cfg.collisions && !side) {
+        collisions(c, A, B.vx, B.vy, B.vz, dt, false);   // (no overlap: a batch's streams share the GPU)
+        if (resolve) {
+            Stage st(c, NCORP_STAGE_COLLIDE);
+            launch_resolve(c, A, B, n, dt);
+            // the drifted box again, if a moonlet's drift changed (the new tree set's control block)
+            launch_bbox_gated(c, B.x, B.y, B.z, n, c->alt.ctl, &c->ctl->n_resolved);
         }
     }
     swap_sets(c);
-    build_tree(c, B, B, A, Cn, n, true, true, nullptr, fused ? dt : 0.0);
+    // The search starts after the keys, together with their sort, whose blocks (on the main stream, at the higher
+    // priority) then take their places first: started beside the keys, its first kernel kept the sort, a
+    // cooperative launch, waiting 120 us at N = 1e6.  With resolution the main stream waits for the search, so
+    // that starts at once.
+    if (side && resolve) fork_search();
+    build_tree(c, B, B, A, Cn, n, true, true, nullptr, fused ? dt : 0.0, [&] {
+        if (side && !resolve) fork_search();
+    });
     if (side && resolve) {
         // The tree above was built beside the search from the unresolved drift.  A step that resolved an
         // impact builds it again from the resolved one; otherwise these launches return at once.

@@ -1075,7 +1075,11 @@ __device__ __forceinline__ float cut_f32(double v) {
 // as an FP32 upper bound, with the velocity in FP32, for the pair
 // prefilter).
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(64) k_leaf_collision(ClimbArgs A) {
+// One block per SM, two of which leave the main stream's key sort its room: it
+// needs a block on every SM at once (blocks of 64 threads, up to sixteen on an
+// SM that other kernels had left free, held it back 19 us at N = 1e5).
+constexpr int LEAF_COL_T = 384;
+__global__ void __launch_bounds__(LEAF_COL_T) k_leaf_collision(ClimbArgs A) {
     if (A.gate && *A.gate == 0) return;
     // the grid barrier counter of the parents' cooperative climb that follows on this stream
     if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->bar_count2 = 0;
@@ -1242,7 +1246,7 @@ void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx
     A.leaves = C.leaves; A.ctl = c->ctl; A.dt = dt; A.cv4 = c->cv4;
     A.rc_given = rc_given;
     A.gate = gate;
-    k_leaf_collision<<<8 * c->num_sms, 64, 0, c->stream>>>(A); c->launches++;
+    k_leaf_collision<<<c->num_sms, LEAF_COL_T, 0, c->stream>>>(A); c->launches++;
     NCORP_CUDA_CHECK(cudaGetLastError());
     const int block = 32 * CLIMB_WARPS_COOP;
     const int grid = coop_grid(c, reinterpret_cast<const void *>(k_climb_collision), block, 0);
