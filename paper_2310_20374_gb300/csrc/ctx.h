@@ -103,6 +103,34 @@ __host__ __device__ inline int near_shares(int E, int m, int n_leaves) {
     return (E + per - 1) / per;
 }
 
+// What a walk starts from, reset by the climb before it: its counters, frontier
+// counts and grid barrier and (gravity) the near field's work counter.
+struct WalkStart {
+    int *fcount = nullptr;     // null: no walk follows
+    int *work = nullptr;
+    int gravity = 0, collisions = 0;
+};
+
+#ifdef __CUDACC__
+// by the threads of one block
+__device__ __forceinline__ void walk_start(const WalkStart &W, Ctrl *ctl) {
+    if (!W.fcount) return;
+    for (int i = threadIdx.x; i <= WALK_MAX_ITERS; i += blockDim.x) W.fcount[i] = 0;
+    if (threadIdx.x == 0) {
+        ctl->n_cp2p = ctl->n_cself = 0;
+        // a walk of both criteria lists the next collision search's pairs; a gravity walk alone does not
+        if (W.gravity) ctl->col_stale = W.collisions ? 0 : 1;
+        ctl->dec_pairs_c = ctl->dec_self_c = 0;
+        if (W.work) *W.work = 0;
+        ctl->n_m2l = ctl->n_p2p = ctl->n_self = ctl->n_near = 0;
+        ctl->dec_pairs = ctl->dec_self = ctl->n_inter = 0;
+        ctl->walk_iters = 0;
+        ctl->bar_walk = 0;
+        ctl->walk_abort[0] = ctl->walk_abort[1] = ctl->walk_abort[2] = 0;
+    }
+}
+#endif
+
 // Grid of a cooperative launch: the given blocks per SM, capped by the
 // context's limit so that the cooperative grids of contexts driven on
 // concurrent streams fit on the device together.
@@ -250,12 +278,14 @@ void launch_iota(ncorp_ctx *c, uint32_t *idx, int n);
 
 // ---- tree.cu ----
 void launch_build(ncorp_ctx *c, const ParticleSet &P, int n, int s, const int *gate = nullptr);
-void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double theta);
+// walk: a gravity walk follows (1), a walk of both criteria (2), none (0)
+void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double theta, int walk);
 void launch_multipoles(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G);
 // rc_given (nullable): each moonlet's R + dt |v| given (the velocities are then not read and the pair
-// test's per-moonlet values are not written); gate (nullable): nothing is done while *gate is 0
+// test's per-moonlet values are not written); gate (nullable): nothing is done while *gate is 0; walk: a
+// collision walk follows
 void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx, const double *vy,
-                            const double *vz, double dt, const double *rc_given = nullptr,
+                            const double *vz, double dt, bool walk, const double *rc_given = nullptr,
                             const int *gate = nullptr);
 
 // ---- walk.cu ----

@@ -629,7 +629,7 @@ void gravity(ncorp_ctx *c, ParticleSet &S, int p, double theta, double t, bool w
         try {
             on_stream(c, c->side2, [&] {
                 Stage st(c, NCORP_STAGE_COLLIDE);
-                launch_climb_collision(c, S, S.vx, S.vy, S.vz, fused_dt, c->cells.rc_spec);
+                launch_climb_collision(c, S, S.vx, S.vy, S.vz, fused_dt, false, c->cells.rc_spec);
                 NCORP_CUDA_CHECK(cudaEventRecord(c->ev_spec, c->stream));
             });
         } catch (...) {
@@ -638,7 +638,7 @@ void gravity(ncorp_ctx *c, ParticleSet &S, int p, double theta, double t, bool w
         }
         c->coop_max = cap;
     }
-    { Stage st(c, NCORP_STAGE_CLIMB); launch_climb_geometry(c, S, G, theta); }
+    { Stage st(c, NCORP_STAGE_CLIMB); launch_climb_geometry(c, S, G, theta, fused ? 2 : 1); }
     NCORP_CUDA_CHECK(cudaEventRecord(c->ev_geo, c->stream));
     NCORP_CUDA_CHECK(cudaStreamWaitEvent(c->side2, c->ev_geo, 0));
     on_stream(c, c->side2, [&] {
@@ -670,7 +670,7 @@ void gravity_standard(ncorp_ctx *c, ParticleSet &S, int n, int p, double theta, 
     c->grav_p = p;
     c->grav_mixed = mixed;
     c->grav_local = false;
-    { Stage st(c, NCORP_STAGE_CLIMB); launch_climb_geometry(c, S, G, theta); }
+    { Stage st(c, NCORP_STAGE_CLIMB); launch_climb_geometry(c, S, G, theta, 0); }
     { Stage st(c, NCORP_STAGE_CLIMB); launch_multipoles(c, S, p, mixed, G); }
     Stage st(c, NCORP_STAGE_EVAL);
     launch_standard(c, S, n, p, mixed, G, external(c, t), want_mutual, c->cfg.n_cb_pre, c->cfg.n_cb_post);
@@ -682,7 +682,7 @@ void gravity_standard(ncorp_ctx *c, ParticleSet &S, int n, int p, double theta, 
 void collisions(ncorp_ctx *c, const ParticleSet &S, const double *vx, const double *vy, const double *vz, double dt,
                 bool wide, const int *gate = nullptr) {
     Stage st(c, NCORP_STAGE_COLLIDE);
-    launch_climb_collision(c, S, vx, vy, vz, dt, nullptr, gate);
+    launch_climb_collision(c, S, vx, vy, vz, dt, true, nullptr, gate);
     launch_walk(c, false, true, gate);
     launch_collide(c, S, vx, vy, vz, dt, wide);
 }
@@ -691,7 +691,7 @@ void collisions(ncorp_ctx *c, const ParticleSet &S, const double *vx, const doub
 // per moonlet.  S's velocities are the ones searched.
 void collisions_standard(ncorp_ctx *c, const ParticleSet &S, int n, double dt) {
     Stage st(c, NCORP_STAGE_COLLIDE);
-    launch_climb_collision(c, S, S.vx, S.vy, S.vz, dt);
+    launch_climb_collision(c, S, S.vx, S.vy, S.vz, dt, false);
     launch_standard_collide(c, S, dt, n, c->cfg.c_cb_pre, c->cfg.c_cb_post);
 }
 

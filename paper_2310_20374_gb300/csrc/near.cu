@@ -24,7 +24,7 @@ struct NearArgs {
     const float4 *hi4, *lo4;
     double G;
     double *nx, *ny, *nz;     // near-field sums per moonlet (tree order), zeroed by the gather
-    int *work;                // items handed out so far (zeroed by the gravity walk's k_walk_init)
+    int *work;                // items handed out so far (zeroed by the geometry climb)
     const Ctrl *ctl;
 };
 

@@ -64,6 +64,7 @@ struct BuildArgs {
     int n, s, cap, chunk;   // chunk: moonlets per block, a multiple of BUILD_T
     int *level, *first, *count, *child0, *nchild, *parent, *arrive, *arrive_m;
     uint32_t *cx, *cy, *cz;
+    int *wcnt, *woff;       // the walk's per-cell counts [cap + 1], zeroed for it
     int *leaves, *leaf_of;  // leaf_of[i] first holds moonlet i's levels, (L0 << 8 | Lmax) or -1
     int *bcount;            // [gridDim.x][BUILD_ROW]: cells of each level the block starts, its leaves, and the leaf
                             // level of its last start (-1: none)
@@ -122,7 +123,10 @@ __global__ void __launch_bounds__(BUILD_T) k_build(BuildArgs A) {
     const unsigned le = 0xffffffffu >> (31 - lane);       // lanes up to this one
     const int *doff = A.ctl->doff;
     // ---- 1. the cells each moonlet starts, and the block's counts
-    for (int i = b * BUILD_T + tid; i < A.cap; i += G * BUILD_T) A.count[i] = A.nchild[i] = 0;
+    for (int i = b * BUILD_T + tid; i <= A.cap; i += G * BUILD_T) {
+        if (i < A.cap) A.count[i] = A.nchild[i] = 0;
+        A.wcnt[i] = A.woff[i] = 0;
+    }
     if (tid < BUILD_COUNTS) s_cnt[tid] = 0;
     if (tid == 0) s_prev = -1;
     __syncthreads();
@@ -296,6 +300,7 @@ void launch_build(ncorp_ctx *c, const ParticleSet &P, int n, int s, const int *g
     A.parent = C.parent; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
     A.arrive = C.arrive; A.arrive_m = C.arrive_m;
     A.leaves = C.leaves; A.leaf_of = C.leaf_of;
+    A.wcnt = c->wl.cnt; A.woff = c->wl.p2p_off;
     A.bcount = C.blocksum; A.ctl = c->ctl;
     // ctl->bar_build was zeroed by k_keys
     const int most = std::min(coop_grid(c, reinterpret_cast<const void *>(k_build), BUILD_T, 0),
@@ -406,6 +411,7 @@ struct ClimbArgs {
     double G, dt, theta;
     double K3;                // (theta_min^5 / (1 - theta_min)^2)^3
     int cap;
+    WalkStart ws;             // the walk that follows
     const double *rc_given;   // collision climb (nullable): each moonlet's R + dt |v| given (tree order)
     const int *gate;          // collision climb (nullable): nothing to do while *gate is 0
 };
@@ -979,6 +985,7 @@ __global__ void __launch_bounds__(32 * CLIMB_WARPS_COOP) k_geometry(ClimbArgs A)
     // warps numbered across the blocks first, so that consecutive work items land on different SMs
     const int gw0 = (threadIdx.x >> 5) * gridDim.x + blockIdx.x, nwarps = (gridDim.x * blockDim.x) >> 5;
     unsigned bar = 0;
+    if (blockIdx.x == 0) walk_start(A.ws, A.ctl);
     const int n_leaves = A.ctl->n_leaves;
     for (int gw = gw0; gw * LEAF_GROUP < n_leaves; gw += nwarps) leaf_gravity_group(A, gw, lane, n_leaves);
     if (!grid_sync(A.ctl, bar)) return;
@@ -1007,7 +1014,7 @@ __global__ void __launch_bounds__(32 * CLIMB_WARPS_COOP) k_geometry(ClimbArgs A)
 }
 
 
-void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double theta) {
+void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double theta, int walk) {
     Cells &C = c->cells;
     ClimbArgs A{};
     A.x = P.x; A.y = P.y; A.z = P.z; A.m = P.m; A.hi4 = P.hi4; A.lo4 = P.lo4;
@@ -1016,6 +1023,12 @@ void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double 
     A.M = C.M; A.sx = C.sx; A.sy = C.sy; A.sz = C.sz; A.rmax = C.rmax; A.rcrit = C.rcrit; A.rho = C.rho;
     A.gh = C.gh; A.gl = C.gl;
     A.Mh = C.Mh; A.leaves = C.leaves; A.ctl = c->ctl; A.G = G; A.theta = theta; A.cap = C.cap;
+    if (walk) {
+        A.ws.fcount = c->wl.front_count;
+        A.ws.work = c->work_counter;
+        A.ws.gravity = 1;
+        A.ws.collisions = walk == 2;
+    }
     {   // K^3, each operation rounded once as on the device (no contraction: products and quotients only)
         const double t2 = theta * theta, t4 = t2 * t2, t5 = t4 * theta, u = 1.0 - theta, u2 = u * u, K = t5 / u2;
         const double K2 = K * K;
@@ -1084,6 +1097,7 @@ __global__ void __launch_bounds__(LEAF_COL_T) k_leaf_collision(ClimbArgs A) {
     // the grid barrier counter of the parents' cooperative climb that follows on this stream
     if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->bar_count2 = 0;
     if (aborted(A.ctl)) return;
+    if (blockIdx.x == 0) walk_start(A.ws, A.ctl);
     const int lane = threadIdx.x & 31;
     const int n_leaves = A.ctl->n_leaves;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
@@ -1234,7 +1248,7 @@ __global__ void __launch_bounds__(32 * CLIMB_WARPS_COOP) k_climb_collision(Climb
 }
 
 void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx, const double *vy,
-                            const double *vz, double dt, const double *rc_given, const int *gate) {
+                            const double *vz, double dt, bool walk, const double *rc_given, const int *gate) {
     Cells &C = c->cells;
     ClimbArgs A{};
     A.x = P.x; A.y = P.y; A.z = P.z; A.R = P.R; A.vx = vx; A.vy = vy; A.vz = vz;
@@ -1244,6 +1258,10 @@ void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx
     A.sx = C.bx; A.sy = C.by; A.sz = C.bz; A.rmax = C.bmax; A.rcrit = C.bcrit;
     A.gh = C.bh; A.gl = C.bl;
     A.leaves = C.leaves; A.ctl = c->ctl; A.dt = dt; A.cv4 = c->cv4;
+    if (walk) {
+        A.ws.fcount = c->wl.front_count;
+        A.ws.collisions = 1;
+    }
     A.rc_given = rc_given;
     A.gate = gate;
     k_leaf_collision<<<c->num_sms, LEAF_COL_T, 0, c->stream>>>(A); c->launches++;

@@ -58,7 +58,6 @@ struct WalkArgs {
     const int *first;
     int2 *m2l_dir;
     int m2l_dir_cap, p2p_dir_cap;
-    int *work;                 // gravity: the near-field kernel's work counter, zeroed by k_walk_init
     Ctrl *ctl;
 };
 
@@ -71,33 +70,6 @@ constexpr int C_FORCED = static_cast<int>(0x80000000u); // x: collisions forced
 constexpr int G_DONE = 1 << 30;                          // x: gravity has decided the pair
 constexpr int C_DONE = 1 << 29;                          // x: the collision criterion has decided the pair
 constexpr int CELL_MASK = (1 << 29) - 1;
-
-// One thread: the root pairs, zeroed frontier counts and counters, and (for
-// gravity) the work counter of the near-field kernel that reads the lists.
-__global__ void k_walk_init(WalkArgs A) {
-    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;
-    const int nd = A.ctl->nd;   // one root pair per disk (a forest's disks never interact)
-    for (int d = 0; d < nd; d++) A.front0[d] = make_int2(d, d);
-    A.ctl->n_cp2p = 0;
-    A.ctl->n_cself = 0;
-    // a walk of both criteria lists the next collision search's pairs; a gravity walk alone does not
-    if (A.gravity) A.ctl->col_stale = A.collisions ? 0 : 1;
-    A.ctl->dec_pairs_c = 0;
-    A.ctl->dec_self_c = 0;
-    for (int i = 1; i <= WALK_MAX_ITERS; i++) A.fcount[i] = 0;
-    A.fcount[0] = nd;
-    if (A.work) *A.work = 0;
-    A.ctl->n_m2l = 0;
-    A.ctl->n_p2p = 0;
-    A.ctl->n_self = 0;
-    A.ctl->n_near = 0;
-    A.ctl->dec_pairs = 0;
-    A.ctl->dec_self = 0;
-    A.ctl->n_inter = 0;
-    A.ctl->walk_iters = 0;
-    A.ctl->bar_count = 0;
-    A.ctl->walk_abort[0] = A.ctl->walk_abort[1] = A.ctl->walk_abort[2] = 0;
-}
 
 __device__ __forceinline__ long long warp_sum_ll(long long v) {
 #pragma unroll
@@ -149,35 +121,19 @@ __device__ __forceinline__ int aggregated_add(int *m2l_ctr, int *p2p_ctr, int ke
 
 // Directed lists from the walk's output (gravity): M2L (A, B) gives A <- B
 // and B <- A grouped by target; leaf pairs give A <- B and B <- A, self
-// leaves A <- A, grouped by target leaf.  Counting sort: counts (warp-
-// aggregated atomics), prefix sums over all blocks (chunk sums, a barrier,
-// chunk scans), scatter (aggregated again: entries of one target in an order
-// set by the atomics).  The frontier buffers, idle after the walk, hold the
-// chunk sums.
+// leaves A <- A, grouped by target leaf.  Counting sort: the walk counted the
+// targets as it emitted the pairs (additions nobody waits for, in generations
+// that wait for loads and barriers; as a pass of its own over the lists the
+// count took 8 us at N = 1e5 and 66 us at 1e6, bound by the L2's atomics); prefix
+// sums over all blocks (chunk sums, a barrier, chunk scans), scatter (warp-
+// aggregated atomics: entries of one target in an order set by the atomics).
+// The frontier buffers, idle after the walk, hold the chunk sums.
 __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
     const int nm = min(A.ctl->n_m2l, A.m2l_cap), np = min(A.ctl->n_p2p, A.p2p_cap),
               ns = min(A.ctl->n_self, A.self_cap);
     const int nc = A.ctl->n_cells + 1, total = nm + np + ns;
     const int lane = threadIdx.x & 31;
     const int wbase = (blockIdx.x * blockDim.x + threadIdx.x - lane), wstride = gridDim.x * blockDim.x;
-    for (int base = wbase; base < total; base += wstride) {
-        const int i = base + lane;
-        int k0 = -1, k1 = -1;
-        if (i < nm) {
-            const int2 e = __ldcg(&A.m2l[i]);
-            k0 = 2 * e.x;
-            k1 = 2 * e.y;
-        } else if (i < nm + np) {
-            const int2 e = __ldcg(&A.p2p[i - nm]);
-            k0 = 2 * e.x + 1;
-            k1 = 2 * e.y + 1;
-        } else if (i < total) {
-            k0 = 2 * __ldcg(&A.self[i - nm - np]) + 1;
-        }
-        aggregated_add(A.cnt, A.p2p_off, k0);
-        aggregated_add(A.cnt, A.p2p_off, k1);
-    }
-    if (!grid_sync(A.ctl, bar)) return;
     // chunk sums of both count arrays
     int *bs = reinterpret_cast<int *>(A.front0);   // [2][gridDim.x]
     const int G = gridDim.x, ch = (nc + G - 1) / G;
@@ -196,7 +152,7 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
             bs[G + blockIdx.x] = tp;
         }
     }
-    if (!grid_sync(A.ctl, bar)) return;
+    if (!grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
     {
         __shared__ int s_items;
         const int n_leaves = A.ctl->n_leaves;
@@ -250,7 +206,7 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
             A.ctl->n_p2p_dir = 2 * np + ns;
         }
     }
-    if (!grid_sync(A.ctl, bar)) return;
+    if (!grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
     for (int base = wbase; base < total; base += wstride) {
         const int i = base + lane;
         int k0 = -1, k1 = -1;
@@ -386,12 +342,259 @@ __device__ __forceinline__ WalkDec walk_decide(const WalkCrit &K, bool grav, int
 
 __device__ __forceinline__ bool is_split(int k) { return k >= O_SPLIT_SELF; }
 
-// One generation of the walk: the pairs cur[0, nf) of generation it, taken
-// a block of WALK_THREADS at a time (warp w of the block takes the w-th 32);
-// outcomes appended to the lists and children pairs to the next frontier.
+// What becomes of a pair of the frontier: its entries in the lists and the k
+// pairs of children that follow it (split: their form, cells c0 .. c0 + nch - 1 of
+// the split cell with flags fx, fy).
+struct WalkOut {
+    int cA, cB;
+    bool m2l, p2p, self, cp2p, cself;
+    int split, c0, nch, k, fx, fy;
+};
+
 // The decision statistics are added to the thread's totals st[5] (gravity:
 // direct pairs, direct self cells, moonlet pairs; collisions: direct pairs,
 // direct self cells).
+template <bool GRAV, bool COL>
+__device__ __forceinline__ WalkOut walk_pair(const WalkArgs &A, bool valid, int2 e, long long *st) {
+    WalkOut o;
+    int cA = 0, cB = 0;
+    bool g_act = false, c_act = false, g_forced = false, c_forced = false;
+    if (valid) {
+        cA = e.x & CELL_MASK;
+        cB = e.y & 0x7fffffff;
+        g_act = GRAV && !(e.x & G_DONE);
+        c_act = COL && !(e.x & C_DONE);
+        g_forced = (e.y & FORCED) != 0;
+        c_forced = (e.x & C_FORCED) != 0;
+    }
+    // every cell field this lane may need, loaded in one round
+    int nA = 0, nB = 0, chA = 0, chB = 0, c0A = 0, c0B = 0;
+    float4 ha = make_float4(0.f, 0.f, 0.f, 0.f), hb = ha, la = ha, lb = ha, ka = ha, kb = ha, ma = ha, mb = ha;
+    double rA = 0.0, rB = 0.0, qA = 0.0, qB = 0.0;
+    if (valid) {
+        nA = __ldg(&A.count[cA]);
+        nB = __ldg(&A.count[cB]);
+        chA = __ldg(&A.nchild[cA]);
+        chB = __ldg(&A.nchild[cB]);
+        c0A = __ldg(&A.child0[cA]);
+        c0B = __ldg(&A.child0[cB]);
+    }
+    if (GRAV && g_act) {
+        ha = __ldg(&A.g.H[cA]);
+        hb = __ldg(&A.g.H[cB]);
+        la = __ldg(&A.g.Lo[cA]);
+        lb = __ldg(&A.g.Lo[cB]);
+        rA = __ldg(&A.g.rcrit[cA]);
+        rB = __ldg(&A.g.rcrit[cB]);
+    }
+    if (COL && c_act) {
+        ka = __ldg(&A.c.H[cA]);
+        kb = __ldg(&A.c.H[cB]);
+        ma = __ldg(&A.c.Lo[cA]);
+        mb = __ldg(&A.c.Lo[cB]);
+        qA = __ldg(&A.c.rcrit[cA]);
+        qB = __ldg(&A.c.rcrit[cB]);
+    }
+    WalkDec gd{O_NONE, false, 0, 0, 0}, cd{O_NONE, false, 0, 0, 0};
+    if (GRAV && g_act) gd = walk_decide(A.g, true, cA, cB, g_forced, nA, nB, chA, chB, ha, la, hb, lb, rA, rB);
+    if (COL && c_act) cd = walk_decide(A.c, false, cA, cB, c_forced, nA, nB, chA, chB, ka, ma, kb, mb, qA, qB);
+    st[0] += gd.dpair;
+    st[1] += gd.dself;
+    st[2] += gd.inter;
+    st[3] += cd.dpair;
+    st[4] += cd.dself;
+    o.cA = cA;
+    o.cB = cB;
+    o.m2l = gd.kind == O_M2L;
+    o.p2p = gd.kind == O_P2P;
+    o.self = gd.kind == O_SELF;
+    o.cp2p = cd.kind == O_P2P;
+    o.cself = cd.kind == O_SELF;
+    // the split: gravity's choice while gravity acts on the pair, else the collision criterion's
+    const bool gs = is_split(gd.kind), cs = is_split(cd.kind);
+    o.split = gs ? gd.kind : (cs ? cd.kind : O_NONE);
+    // flags of the children: each criterion that split goes on, with its forced state
+    o.fx = o.fy = 0;
+    if (o.split != O_NONE) {
+        if (!gs) o.fx |= G_DONE;
+        else if (gd.child_forced) o.fy |= FORCED;
+        if (!cs) o.fx |= C_DONE;
+        else if (cd.child_forced) o.fx |= C_FORCED;
+    }
+    o.c0 = o.nch = o.k = 0;
+    if (o.split == O_SPLIT_SELF) {
+        o.c0 = c0A;
+        o.nch = chA;
+        o.k = chA * (chA + 1) / 2;
+    } else if (o.split == O_SPLIT_A) {
+        o.c0 = c0A;
+        o.nch = o.k = chA;
+    } else if (o.split == O_SPLIT_B) {
+        o.c0 = c0B;
+        o.nch = o.k = chB;
+    }
+    return o;
+}
+
+// The k pairs of children of an outcome, through put(index, pair).
+template <class F>
+__device__ __forceinline__ void walk_children(const WalkOut &o, F put) {
+    int q = 0;
+    if (o.split == O_SPLIT_SELF) {
+        for (int a = 0; a < o.nch; a++)
+            for (int b = a; b < o.nch; b++) put(q++, make_int2((o.c0 + a) | o.fx, (o.c0 + b) | o.fy));
+    } else if (o.split == O_SPLIT_A) {
+        for (int a = 0; a < o.nch; a++) put(q++, make_int2((o.c0 + a) | o.fx, o.cB | o.fy));
+    } else {
+        for (int b = 0; b < o.nch; b++) put(q++, make_int2(o.cA | o.fx, (o.c0 + b) | o.fy));
+    }
+}
+
+// An outcome's entries written to their slots of the lists (M2L, direct pairs,
+// self leaves; the collision criterion's pairs and self leaves), and the
+// targets counted; false if a list is full (its error is set).
+__device__ __forceinline__ bool walk_emit(const WalkArgs &A, const WalkOut &o, const int slot[5]) {
+    int err = 0;
+    if (o.m2l) {
+        if (slot[0] < A.m2l_cap) {
+            A.m2l[slot[0]] = make_int2(o.cA, o.cB);
+            atomicAdd(&A.cnt[o.cA], 1);
+            atomicAdd(&A.cnt[o.cB], 1);
+        } else err = ERR_M2L;
+    }
+    if (o.p2p) {
+        if (slot[1] < A.p2p_cap) {
+            A.p2p[slot[1]] = make_int2(o.cA, o.cB);
+            atomicAdd(&A.p2p_off[o.cA], 1);
+            atomicAdd(&A.p2p_off[o.cB], 1);
+        } else err = ERR_P2P;
+    }
+    if (o.self) {
+        if (slot[2] < A.self_cap) {
+            A.self[slot[2]] = o.cA;
+            atomicAdd(&A.p2p_off[o.cA], 1);
+        } else err = ERR_P2P;
+    }
+    if (o.cp2p) {
+        if (slot[3] < A.cp2p_cap) A.cp2p[slot[3]] = make_int2(o.cA, o.cB);
+        else err = ERR_P2P;
+    }
+    if (o.cself) {
+        if (slot[4] < A.cself_cap) A.cself[slot[4]] = o.cA;
+        else err = ERR_P2P;
+    }
+    if (err) atomicOr(&A.ctl->err, err);
+    return err == 0;
+}
+
+// The walk's head: one block takes the generations from the roots on as long
+// as they fit its shared memory.  A generation costs it the cells' loads and
+// two block barriers, about 1.5 us; among all blocks the frontier's way through
+// memory, the reservations' atomics and the grid barrier make it 4 us, and
+// the first five generations of a large tree hold a few hundred pairs.  Leaves
+// the next generation's pairs in the frontier buffer and its number in
+// ctl->walk_head (-1: a list was full).  A launch of its own: with the head's
+// shared memory in every block of the walk, the SMs would not take the walk's blocks
+// beside those of the kernels on the other streams (150 us of the step at N = 1e6).
+// Head and walk in the step at N = 1e5, with the resets moved into the climb and
+// the targets counted at emission: collisions 78 -> 71 us, gravity 135 -> 118.
+constexpr int HEAD_CAP = 1024, HEAD_THREADS = 512;
+
+struct WalkHead {
+    int2 q[2][HEAD_CAP];
+    int n[5];              // entries of the five lists
+    int next[3], bad[3];   // of generation g in slot g mod 3 (a slot is cleared a generation before its use, when
+                           // every thread has read what it held)
+};
+
+// The threads' decision statistics (walk_pair) added to the walk's: one atomic per block and counter.
+template <int WARPS>
+__device__ __forceinline__ void walk_stats(const WalkArgs &A, const long long st[5], long long (*s_stat)[5]) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 5; k++) {
+        const long long v = warp_sum_ll(st[k]);
+        if (lane == 0) s_stat[w][k] = v;
+    }
+    __syncthreads();
+    if (threadIdx.x < 5) {
+        long long v = 0;
+#pragma unroll
+        for (int ww = 0; ww < WARPS; ww++) v += s_stat[ww][threadIdx.x];
+        long long *dst = threadIdx.x == 0 ? &A.ctl->dec_pairs
+                       : threadIdx.x == 1 ? &A.ctl->dec_self
+                       : threadIdx.x == 2 ? &A.ctl->n_inter
+                       : threadIdx.x == 3 ? &A.ctl->dec_pairs_c : &A.ctl->dec_self_c;
+        if (v) atomicAdd(reinterpret_cast<unsigned long long *>(dst), static_cast<unsigned long long>(v));
+    }
+}
+
+template <bool GRAV, bool COL>
+__global__ void __launch_bounds__(HEAD_THREADS) k_walk_head(WalkArgs A) {
+    __shared__ WalkHead H;
+    __shared__ long long s_stat[HEAD_THREADS / 32][5];
+    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;
+    long long st[5] = {0, 0, 0, 0, 0};
+    const int tid = threadIdx.x;
+    int nf = A.ctl->nd;
+    if (tid < 5) H.n[tid] = 0;
+    if (tid == 0) H.next[0] = H.bad[0] = 0;
+    for (int d = tid; d < nf; d += HEAD_THREADS) H.q[0][d] = make_int2(d, d);   // (nd <= 256 <= HEAD_CAP)
+    __syncthreads();
+    int it = 0;
+    bool bad = false;
+    while (nf > 0 && it < WALK_MAX_ITERS) {
+        const int g = it % 3, g1 = (it + 1) % 3;
+        const int2 *cur = H.q[it & 1];
+        int2 *nxt = H.q[(it + 1) & 1], *out = ((it + 1) & 1) ? A.front1 : A.front0;
+        if (tid == 0) H.next[g1] = H.bad[g1] = 0;
+        for (int i = tid; i < nf; i += HEAD_THREADS) {
+            const WalkOut o = walk_pair<GRAV, COL>(A, true, cur[i], st);
+            int slot[5];
+            slot[0] = o.m2l ? atomicAdd(&H.n[0], 1) : 0;
+            slot[1] = o.p2p ? atomicAdd(&H.n[1], 1) : 0;
+            slot[2] = o.self ? atomicAdd(&H.n[2], 1) : 0;
+            slot[3] = o.cp2p ? atomicAdd(&H.n[3], 1) : 0;
+            slot[4] = o.cself ? atomicAdd(&H.n[4], 1) : 0;
+            if (!walk_emit(A, o, slot)) H.bad[g] = 1;
+            if (o.k > 0) {
+                const int at = atomicAdd(&H.next[g], o.k);
+                if (at + o.k > A.front_cap) {
+                    atomicOr(&A.ctl->err, ERR_FRONTIER);
+                    H.bad[g] = 1;
+                } else {
+                    walk_children(o, [&](int j, int2 e) {
+                        if (at + j < HEAD_CAP) nxt[at + j] = e;
+                        else out[at + j] = e;
+                    });
+                }
+            }
+        }
+        __syncthreads();
+        nf = H.next[g];
+        bad = H.bad[g] != 0;
+        it++;
+        if (bad || nf > HEAD_CAP) {
+            for (int i = tid; i < min(nf, HEAD_CAP); i += HEAD_THREADS) out[i] = nxt[i];
+            break;
+        }
+    }
+    __syncthreads();
+    if (tid == 0) {
+        A.fcount[it] = bad ? 0 : nf;
+        A.ctl->n_m2l = H.n[0];
+        A.ctl->n_p2p = H.n[1];
+        A.ctl->n_self = H.n[2];
+        A.ctl->n_cp2p = H.n[3];
+        A.ctl->n_cself = H.n[4];
+        A.ctl->walk_head = bad ? -1 : it;
+    }
+    walk_stats<HEAD_THREADS / 32>(A, st, s_stat);
+}
+
+// One generation of the walk: the pairs cur[0, nf) of generation it, taken
+// a block of WALK_THREADS at a time (warp w of the block takes the w-th 32);
+// outcomes appended to the lists and children pairs to the next frontier.
 template <bool GRAV, bool COL>
 __device__ __forceinline__ void walk_generation(const WalkArgs &A, int it, int nf, long long *st, WalkSlots &S) {
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -402,84 +605,12 @@ __device__ __forceinline__ void walk_generation(const WalkArgs &A, int it, int n
     for (int bbase = blockIdx.x * WALK_THREADS; bbase < nf; bbase += gridDim.x * WALK_THREADS) {
         const int i = bbase + w * 32 + lane;
         const bool valid = i < nf;
-        int cA = 0, cB = 0;
-        bool g_act = false, c_act = false, g_forced = false, c_forced = false;
-        if (valid) {
-            const int2 e = __ldcg(&cur[i]);
-            cA = e.x & CELL_MASK;
-            cB = e.y & 0x7fffffff;
-            g_act = GRAV && !(e.x & G_DONE);
-            c_act = COL && !(e.x & C_DONE);
-            g_forced = (e.y & FORCED) != 0;
-            c_forced = (e.x & C_FORCED) != 0;
-        }
-        // every cell field this lane may need, loaded in one round
-        int nA = 0, nB = 0, chA = 0, chB = 0, c0A = 0, c0B = 0;
-        float4 ha = make_float4(0.f, 0.f, 0.f, 0.f), hb = ha, la = ha, lb = ha, ka = ha, kb = ha, ma = ha, mb = ha;
-        double rA = 0.0, rB = 0.0, qA = 0.0, qB = 0.0;
-        if (valid) {
-            nA = __ldg(&A.count[cA]);
-            nB = __ldg(&A.count[cB]);
-            chA = __ldg(&A.nchild[cA]);
-            chB = __ldg(&A.nchild[cB]);
-            c0A = __ldg(&A.child0[cA]);
-            c0B = __ldg(&A.child0[cB]);
-        }
-        if (GRAV && g_act) {
-            ha = __ldg(&A.g.H[cA]);
-            hb = __ldg(&A.g.H[cB]);
-            la = __ldg(&A.g.Lo[cA]);
-            lb = __ldg(&A.g.Lo[cB]);
-            rA = __ldg(&A.g.rcrit[cA]);
-            rB = __ldg(&A.g.rcrit[cB]);
-        }
-        if (COL && c_act) {
-            ka = __ldg(&A.c.H[cA]);
-            kb = __ldg(&A.c.H[cB]);
-            ma = __ldg(&A.c.Lo[cA]);
-            mb = __ldg(&A.c.Lo[cB]);
-            qA = __ldg(&A.c.rcrit[cA]);
-            qB = __ldg(&A.c.rcrit[cB]);
-        }
-        WalkDec gd{O_NONE, false, 0, 0, 0}, cd{O_NONE, false, 0, 0, 0};
-        if (GRAV && g_act) gd = walk_decide(A.g, true, cA, cB, g_forced, nA, nB, chA, chB, ha, la, hb, lb, rA, rB);
-        if (COL && c_act) cd = walk_decide(A.c, false, cA, cB, c_forced, nA, nB, chA, chB, ka, ma, kb, mb, qA, qB);
-        st[0] += gd.dpair;
-        st[1] += gd.dself;
-        st[2] += gd.inter;
-        st[3] += cd.dpair;
-        st[4] += cd.dself;
-        const int emit_m2l = gd.kind == O_M2L, emit_p2p = gd.kind == O_P2P, emit_self = gd.kind == O_SELF;
-        const int emit_cp2p = cd.kind == O_P2P, emit_cself = cd.kind == O_SELF;
-        // the split: gravity's choice while gravity acts on the pair, else the collision criterion's
-        const bool gs = is_split(gd.kind), cs = is_split(cd.kind);
-        const int split = gs ? gd.kind : (cs ? cd.kind : O_NONE);
-        // flags of the children: each criterion that split goes on, with its forced state
-        int fx = 0, fy = 0;
-        if (split != O_NONE) {
-            if (!gs) fx |= G_DONE;
-            else if (gd.child_forced) fy |= FORCED;
-            if (!cs) fx |= C_DONE;
-            else if (cd.child_forced) fx |= C_FORCED;
-        }
-        int c0 = 0, nch = 0, k = 0;
-        if (split == O_SPLIT_SELF) {
-            c0 = c0A;
-            nch = chA;
-            k = nch * (nch + 1) / 2;
-        } else if (split == O_SPLIT_A) {
-            c0 = c0A;
-            nch = chA;
-            k = nch;
-        } else if (split == O_SPLIT_B) {
-            c0 = c0B;
-            nch = chB;
-            k = nch;
-        }
+        const WalkOut o = walk_pair<GRAV, COL>(A, valid, valid ? __ldcg(&cur[i]) : make_int2(0, 0), st);
+        const int k = o.k;
         // outputs: the block's warps reserve their slots together, one atomic per list
-        const unsigned bm = __ballot_sync(0xffffffffu, emit_m2l), bp = __ballot_sync(0xffffffffu, emit_p2p),
-                       bs = __ballot_sync(0xffffffffu, emit_self), bcp = __ballot_sync(0xffffffffu, emit_cp2p),
-                       bcs = __ballot_sync(0xffffffffu, emit_cself);
+        const unsigned bm = __ballot_sync(0xffffffffu, o.m2l), bp = __ballot_sync(0xffffffffu, o.p2p),
+                       bs = __ballot_sync(0xffffffffu, o.self), bcp = __ballot_sync(0xffffffffu, o.cp2p),
+                       bcs = __ballot_sync(0xffffffffu, o.cself);
         int kin = k;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -514,48 +645,17 @@ __device__ __forceinline__ void walk_generation(const WalkArgs &A, int it, int n
             for (int ww = 0; ww < WALK_WARPS; ww++) S.base[ww][q] += b0;
         }
         __syncthreads();
-        const int base_m = S.base[w][0], base_p = S.base[w][1], base_s = S.base[w][2], base_f = S.base[w][3],
-                  base_cp = S.base[w][4], base_cs = S.base[w][5];
         const unsigned lt = (1u << lane) - 1u;
-        if (emit_m2l) {
-            const int slot = base_m + __popc(bm & lt);
-            if (slot < A.m2l_cap) A.m2l[slot] = make_int2(cA, cB);
-            else { atomicOr(&A.ctl->err, ERR_M2L); A.ctl->walk_abort[it % 3] = 1; }
-        }
-        if (emit_p2p) {
-            const int slot = base_p + __popc(bp & lt);
-            if (slot < A.p2p_cap) A.p2p[slot] = make_int2(cA, cB);
-            else { atomicOr(&A.ctl->err, ERR_P2P); A.ctl->walk_abort[it % 3] = 1; }
-        }
-        if (emit_self) {
-            const int slot = base_s + __popc(bs & lt);
-            if (slot < A.self_cap) A.self[slot] = cA;
-            else { atomicOr(&A.ctl->err, ERR_P2P); A.ctl->walk_abort[it % 3] = 1; }
-        }
-        if (emit_cp2p) {
-            const int slot = base_cp + __popc(bcp & lt);
-            if (slot < A.cp2p_cap) A.cp2p[slot] = make_int2(cA, cB);
-            else { atomicOr(&A.ctl->err, ERR_P2P); A.ctl->walk_abort[it % 3] = 1; }
-        }
-        if (emit_cself) {
-            const int slot = base_cs + __popc(bcs & lt);
-            if (slot < A.cself_cap) A.cself[slot] = cA;
-            else { atomicOr(&A.ctl->err, ERR_P2P); A.ctl->walk_abort[it % 3] = 1; }
-        }
+        const int slot[5] = {S.base[w][0] + __popc(bm & lt), S.base[w][1] + __popc(bp & lt), S.base[w][2] + __popc(bs & lt),
+                             S.base[w][4] + __popc(bcp & lt), S.base[w][5] + __popc(bcs & lt)};
+        if (!walk_emit(A, o, slot)) A.ctl->walk_abort[it % 3] = 1;
         if (k > 0) {
-            int slot = base_f + kin - k;
-            if (slot + k > A.front_cap) {
+            const int at = S.base[w][3] + kin - k;
+            if (at + k > A.front_cap) {
                 atomicOr(&A.ctl->err, ERR_FRONTIER);
                 A.ctl->walk_abort[it % 3] = 1;
             } else {
-                if (split == O_SPLIT_SELF) {
-                    for (int a = 0; a < nch; a++)
-                        for (int b = a; b < nch; b++) nxt[slot++] = make_int2((c0 + a) | fx, (c0 + b) | fy);
-                } else if (split == O_SPLIT_A) {
-                    for (int a = 0; a < nch; a++) nxt[slot++] = make_int2((c0 + a) | fx, cB | fy);
-                } else {
-                    for (int b = 0; b < nch; b++) nxt[slot++] = make_int2(cA | fx, (c0 + b) | fy);
-                }
+                walk_children(o, [&](int j, int2 e) { nxt[at + j] = e; });
             }
         }
     }
@@ -567,49 +667,28 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs A) {
     __shared__ WalkSlots S;
     __shared__ long long s_stat[WALK_WARPS][5];
     if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;   // (every block, before the first barrier)
-    if (A.gravity) {   // list counters, zeroed before the first barrier of the walk
-        const int nc = A.ctl->n_cells + 1;
-        for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < nc; i += gridDim.x * blockDim.x) {
-            A.cnt[i] = 0;
-            A.p2p_off[i] = 0;
-        }
-    }
     volatile int *vcount = A.fcount;
     unsigned bar = 0;
-    int it = 0;
     long long st[5] = {0, 0, 0, 0, 0};   // decision statistics of this thread's pairs
-    for (; it < WALK_MAX_ITERS; it++) {
-        const int nf = min(vcount[it], A.front_cap);
-        if (nf == 0) break;
-        if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->walk_abort[(it + 1) % 3] = 0;   // slot of the next generation
-        walk_generation<GRAV, COL>(A, it, nf, st, S);
-        if (!grid_sync(A.ctl, bar)) return;
-        // overflow in this generation (slot it mod 3: identical for every block after the barrier)
-        if (((volatile int *)A.ctl->walk_abort)[it % 3]) { it++; break; }
-    }
-    {   // the statistics: one atomic per block and counter
-        const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-#pragma unroll
-        for (int k = 0; k < 5; k++) {
-            const long long v = warp_sum_ll(st[k]);
-            if (lane == 0) s_stat[w][k] = v;
+    int it = A.ctl->walk_head;
+    const bool head_bad = it < 0;
+    if (head_bad) it = 0;
+    else
+        for (; it < WALK_MAX_ITERS; it++) {
+            const int nf = min(vcount[it], A.front_cap);
+            if (nf == 0) break;
+            if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->walk_abort[(it + 1) % 3] = 0;   // slot of the next generation
+            walk_generation<GRAV, COL>(A, it, nf, st, S);
+            if (!grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
+            // overflow in this generation (slot it mod 3: identical for every block after the barrier)
+            if (((volatile int *)A.ctl->walk_abort)[it % 3]) { it++; break; }
         }
-        __syncthreads();
-        if (threadIdx.x < 5) {
-            long long v = 0;
-#pragma unroll
-            for (int ww = 0; ww < WALK_WARPS; ww++) v += s_stat[ww][threadIdx.x];
-            long long *dst = threadIdx.x == 0 ? &A.ctl->dec_pairs
-                           : threadIdx.x == 1 ? &A.ctl->dec_self
-                           : threadIdx.x == 2 ? &A.ctl->n_inter
-                           : threadIdx.x == 3 ? &A.ctl->dec_pairs_c : &A.ctl->dec_self_c;
-            if (v) atomicAdd(reinterpret_cast<unsigned long long *>(dst), static_cast<unsigned long long>(v));
-        }
-        // the collision statistics' copies below read every block's totals
-        if (A.collisions && !grid_sync(A.ctl, bar)) return;
-    }
+    walk_stats<WALK_WARPS>(A, st, s_stat);
+    // the collision statistics' copies below read every block's totals
+    if (A.collisions && !grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
     // the generation count and the barrier snapshot are the same in every block
-    if (A.gravity && it < WALK_MAX_ITERS && !((volatile int *)A.ctl->walk_abort)[(it + 2) % 3]) walk_lists(A, s_tmp, bar);
+    if (A.gravity && !head_bad && it < WALK_MAX_ITERS && !((volatile int *)A.ctl->walk_abort)[(it + 2) % 3])
+        walk_lists(A, s_tmp, bar);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (A.gravity) A.ctl->walk_iters = it;
         if (A.collisions) {
@@ -636,6 +715,7 @@ static WalkCrit walk_crit(const ncorp_ctx *c, bool gravity) {
     return K;
 }
 
+// The counters were reset by the climb that precedes the walk (walk_start in ctx.h).
 void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     Cells &C = c->cells;
     WalkLists &W = c->wl;
@@ -655,19 +735,23 @@ void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     A.cnt = W.cnt; A.offs = W.offs; A.cursor = W.cursor; A.p2p_off = W.p2p_off; A.p2p_src = W.p2p_src;
     A.near_items = W.near_items; A.near_cap = W.near_cap;
     A.m2l_dir = W.m2l_dir; A.m2l_dir_cap = W.m2l_dir_cap; A.p2p_dir_cap = W.p2p_dir_cap;
-    A.work = gravity ? c->work_counter : nullptr;
     A.ctl = c->ctl;
-    k_walk_init<<<1, 1, 0, c->stream>>>(A); c->launches++;
-    NCORP_CUDA_CHECK(cudaGetLastError());
     const void *kern = gravity && collisions ? reinterpret_cast<const void *>(k_walk<true, true>)
                      : gravity              ? reinterpret_cast<const void *>(k_walk<true, false>)
                                             : reinterpret_cast<const void *>(k_walk<false, true>);
     int per_sm = 0;
     NCORP_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WALK_THREADS, 0));
     if (per_sm < 1) per_sm = 1;
+    // (four blocks per SM take 300 us instead of 375 alone at N = 1e6, but in a step the launch waits for room
+    // beside the multipoles: the step 2610 -> 2910 us)
     if (per_sm > 2) per_sm = 2;
     // about one block per 640 moonlets (frontiers peak near a third of n pairs), 32 to the cooperative limit
     const int grid = std::min(coop_blocks(c, per_sm), std::max(32, c->cur_n / 640));
+    if (gravity && collisions) k_walk_head<true, true><<<1, HEAD_THREADS, 0, c->stream>>>(A);
+    else if (gravity) k_walk_head<true, false><<<1, HEAD_THREADS, 0, c->stream>>>(A);
+    else k_walk_head<false, true><<<1, HEAD_THREADS, 0, c->stream>>>(A);
+    c->launches++;
+    NCORP_CUDA_CHECK(cudaGetLastError());
     void *args[] = {&A};
     NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(WALK_THREADS), args, 0, c->stream));
     c->launches++;
