@@ -592,8 +592,8 @@ __global__ void k_unpack_pairs(const uint64_t *__restrict__ packed, int64_t *__r
 
 void launch_sort_pairs(ncorp_ctx *c, int count) {
     if (count <= 0) return;
-    launch_iota(c, c->pair_idx, count);
-    radix_sort_u64(c, c->pairs, c->pair_idx, c->pairs_alt, c->pair_idx_alt, count, 64);
+    if (count > SAMPLE_SORT_MAX) launch_iota(c, c->pair_idx, count);
+    sort_u64(c, c->pairs, c->pair_idx, c->pairs_alt, c->pair_idx_alt, count, 64);
 }
 
 void launch_unpack_pairs(ncorp_ctx *c, const uint64_t *packed, int64_t *out, int count) {

@@ -20,52 +20,21 @@ namespace ncorp {
 // ---------------------------------------------------------------------------
 // bounding box
 // ---------------------------------------------------------------------------
-// One block per SM at most; every thread folds its moonlets into running
-// minima and maxima of the order-preserving integer images of the
-// coordinates (integer min/max, no FP64 instruction), the block reduces them
-// in shared memory and adds one atomic per bound.  A coordinate whose
-// exponent field is all ones (infinite or NaN) sets ERR_NONFINITE.  With a
-// gate, the launch does nothing while *gate is 0.
-__global__ void __launch_bounds__(256) k_bbox(const double *__restrict__ x, const double *__restrict__ y,
-                                              const double *__restrict__ z, int n, Ctrl *ctl,
-                                              const int *gate = nullptr) {
+// A coordinate folded into a thread's bounds (order-preserving integer images).
+__device__ __forceinline__ void fold_coordinate(double v, unsigned long long &lo, unsigned long long &hi, bool &bad) {
+    const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(v));
+    bad |= (u & 0x7ff0000000000000ull) == 0x7ff0000000000000ull;
+    const unsigned long long e = ord_encode(v);
+    lo = e < lo ? e : lo;
+    hi = e > hi ? e : hi;
+}
+
+// The threads' bounds (order-preserving integer images), and their signs of a coordinate that is not finite, added
+// to the box: every thread of a block of at most 256.
+__device__ __forceinline__ void fold_box(unsigned long long lo[3], unsigned long long hi[3], bool bad, Ctrl *ctl) {
     __shared__ unsigned long long s_b[6][8];
     __shared__ int s_bad;
-    if ((gate && *gate == 0) || aborted(ctl)) return;
-    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
-    bool bad = false;
-    if (ctl->disk_of) {   // a forest: every disk's own box
-        const int lane = threadIdx.x & 31;
-        for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += gridDim.x * blockDim.x) {
-            const int i = base + lane;
-            const bool valid = i < n;
-            unsigned long long l[3] = {~0ull, ~0ull, ~0ull}, h[3] = {0ull, 0ull, 0ull};
-            if (valid) {
-                const double v[3] = {x[i], y[i], z[i]};
-#pragma unroll
-                for (int k = 0; k < 3; k++) {
-                    const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(v[k]));
-                    bad |= (u & 0x7ff0000000000000ull) == 0x7ff0000000000000ull;
-                    l[k] = h[k] = ord_encode(v[k]);
-                }
-            }
-            fold_disk_box(ctl, valid ? ctl->disk_of[i] : 0, valid, l, h);
-        }
-        if (bad) atomicOr(&ctl->err, ERR_NONFINITE);
-        return;
-    }
     if (threadIdx.x == 0) s_bad = 0;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const double v[3] = {x[i], y[i], z[i]};
-#pragma unroll
-        for (int k = 0; k < 3; k++) {
-            const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(v[k]));
-            bad |= (u & 0x7ff0000000000000ull) == 0x7ff0000000000000ull;
-            const unsigned long long e = ord_encode(v[k]);
-            lo[k] = e < lo[k] ? e : lo[k];
-            hi[k] = e > hi[k] ? e : hi[k];
-        }
-    }
 #pragma unroll
     for (int k = 0; k < 3; k++)
 #pragma unroll
@@ -96,6 +65,46 @@ __global__ void __launch_bounds__(256) k_bbox(const double *__restrict__ x, cons
         else atomicMax(&ctl->bbox[k], r);
     }
     if (threadIdx.x == 0 && s_bad) atomicOr(&ctl->err, ERR_NONFINITE);
+}
+
+// One block per SM at most; every thread folds its moonlets into running
+// minima and maxima of the order-preserving integer images of the
+// coordinates (integer min/max, no FP64 instruction), the block reduces them
+// in shared memory and adds one atomic per bound.  A coordinate whose
+// exponent field is all ones (infinite or NaN) sets ERR_NONFINITE.  With a
+// gate, the launch does nothing while *gate is 0.
+__global__ void __launch_bounds__(256) k_bbox(const double *__restrict__ x, const double *__restrict__ y,
+                                              const double *__restrict__ z, int n, Ctrl *ctl,
+                                              const int *gate = nullptr) {
+    if ((gate && *gate == 0) || aborted(ctl)) return;
+    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
+    bool bad = false;
+    if (ctl->disk_of) {   // a forest: every disk's own box
+        const int lane = threadIdx.x & 31;
+        for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += gridDim.x * blockDim.x) {
+            const int i = base + lane;
+            const bool valid = i < n;
+            unsigned long long l[3] = {~0ull, ~0ull, ~0ull}, h[3] = {0ull, 0ull, 0ull};
+            if (valid) {
+                const double v[3] = {x[i], y[i], z[i]};
+#pragma unroll
+                for (int k = 0; k < 3; k++) {
+                    const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(v[k]));
+                    bad |= (u & 0x7ff0000000000000ull) == 0x7ff0000000000000ull;
+                    l[k] = h[k] = ord_encode(v[k]);
+                }
+            }
+            fold_disk_box(ctl, valid ? ctl->disk_of[i] : 0, valid, l, h);
+        }
+        if (bad) atomicOr(&ctl->err, ERR_NONFINITE);
+        return;
+    }
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const double v[3] = {x[i], y[i], z[i]};
+#pragma unroll
+        for (int k = 0; k < 3; k++) fold_coordinate(v[k], lo[k], hi[k], bad);
+    }
+    fold_box(lo, hi, bad, ctl);
 }
 
 // ---------------------------------------------------------------------------
@@ -516,10 +525,234 @@ __global__ void __launch_bounds__(RS_T) k_radix(RadixArgs A) {
     radix_body(A, bar);
 }
 
-// Sorts keys/vals in place (the alt buffers are scratch); `bits` low bits of
-// the key are significant (rounded up to an even number of 8-bit passes, so
-// the result ends in the input buffers).  bar_zeroed: the caller's stream has
-// already zeroed ctl->bar_count since the last cooperative kernel.
+// ---------------------------------------------------------------------------
+// Sample sort of up to SS_MAX_N keys whose values are 0 .. n - 1 (so the
+// order of equal keys is the order of places, and every (key, place) differs):
+// one cooperative launch with three grid barriers in place of the radix
+// sort's nine, bound by their latency and the loads between them.
+//   1. S = 8 B samples, spread evenly over the input in runs of four (a run is
+//      one sector), are ranked by counting, every block a share of them; every
+//      eighth of the ranked samples bounds a bucket;
+//   2. every key finds its bucket by binary search in shared memory and
+//      takes a place in its block's part of the bucket (an atomic in shared
+//      memory, one reservation per block and bucket); bucket and place are
+//      kept in the value array, whose input is known;
+//   3. keys and values move to their buckets in the scratch arrays;
+//   4. a block takes a bucket into shared memory and ranks every key by
+//      counting the smaller ones (three instructions a pair; equal keys, seen when
+//      two keys claim one rank, are ranked again with their places).
+// Buckets hold 64 keys on average for few keys (so that they spread over the
+// chip), up to 256 from 16384 keys on (the counting grows with the bucket,
+// the search and the sample ranking with their number, at most 1024).
+// With eight samples a bucket the largest of a thousand buckets is about 2.7
+// averages; a bucket above SS_CAP (keys that differ only between the samples)
+// sends the call to the radix sort, in the same launch.  Measured: N = 4e3 9 us,
+// 6.5e4 17, 1.2e5 26, 2e5 44 (ranks 10, search 9, moves 4, buckets 13, barriers), 5.2e5 102; the radix sort's
+// eight passes take 51, 84, 101, 117 and 149.  Past SS_MAX_N the buckets' counting, which grows with their size,
+// would overtake the radix passes.
+// ---------------------------------------------------------------------------
+constexpr int SS_T = RS_T, SS_BUCKETS = 1024, SS_OVER = 8, SS_CAP = 2048, SS_TARGETS = 4, SS_STAGE = 4096;
+constexpr int SS_MAX_N = SAMPLE_SORT_MAX;   // v0 holds bucket << 20 | place; 12 fraction bits of the sampling stride
+static_assert(SS_MAX_N <= 1 << 19 && SS_BUCKETS <= 1 << 11, "packing of bucket and place");
+
+struct SampleScratch {
+    unsigned long long skey[SS_BUCKETS];   // the buckets' first samples, from bucket 1 on
+    unsigned spos[SS_BUCKETS];
+    int count[SS_BUCKETS];                 // keys of a bucket
+};
+
+struct SampleArgs {
+    RadixArgs radix;   // the arrays, and the radix sort for inputs the samples do not split
+    SampleScratch *scr;
+    int buckets;
+    long long *order;  // nullable: the values as 64-bit integers, in place of v0
+};
+
+__host__ __device__ inline int sample_buckets(int n) {
+    const int fine = n / 64 < 256 ? n / 64 : 256, b = n / 256 > fine ? n / 256 : fine;
+    return b < 1 ? 1 : (b > SS_BUCKETS ? SS_BUCKETS : b);
+}
+
+// Place of sample j of S in an input of n keys (n >= 4 S / 4 = S; S a multiple of four).
+__device__ __forceinline__ int sample_place(int j, unsigned stride) {
+    return 4 * static_cast<int>((static_cast<unsigned>(j >> 2) * stride) >> 12) + (j & 3);
+}
+
+struct SampleSplit {
+    unsigned long long key[SS_BUCKETS];
+    unsigned pos[SS_BUCKETS];
+    int cnt[SS_BUCKETS];       // keys of the block in each bucket, then the block's first place in it
+};
+struct SampleBucket {
+    unsigned long long key[SS_CAP];
+    unsigned val[SS_CAP];
+    int claim[SS_CAP];
+};
+
+__global__ void __launch_bounds__(SS_T) k_sample(SampleArgs A) {
+    __shared__ union {
+        unsigned long long sample[SS_STAGE];
+        SampleSplit split;
+        SampleBucket bucket;
+    } U;
+    __shared__ int s_start[SS_BUCKETS + 1];
+    __shared__ int s_warp[33];
+    const RadixArgs &R = A.radix;
+    // every block returns before the first barrier (an aborted step's keys are never used)
+    if ((R.gate && *R.gate == 0) || aborted(R.ctl)) return;
+    const int tid = threadIdx.x, lane = tid & 31, w = tid >> 5, G = gridDim.x, b = blockIdx.x;
+    const int n = R.n, B = A.buckets, S = SS_OVER * B;
+    unsigned bar = 0;
+    // ---- 1. the samples ranked
+    if (b == 0)
+        for (int i = tid; i < B; i += SS_T) A.scr->count[i] = 0;
+    if (B > 1) {
+        const unsigned stride = (static_cast<unsigned>(n / 4) << 12) / static_cast<unsigned>(S / 4);
+        constexpr int PER_BLOCK = SS_T / 32 * SS_TARGETS;
+        for (int r0 = 0; r0 < S; r0 += G * PER_BLOCK) {
+            if (r0 + b * SS_TARGETS >= S) break;   // (the same for the whole block)
+            const int i0 = r0 + (w * G + b) * SS_TARGETS;   // warps numbered across the blocks; S % SS_TARGETS == 0
+            const bool act = i0 < S;
+            unsigned long long t[SS_TARGETS];
+            int acc[SS_TARGETS];
+#pragma unroll
+            for (int u = 0; u < SS_TARGETS; u++) {
+                t[u] = act ? R.k0[sample_place(i0 + u, stride)] : 0ull;
+                acc[u] = 0;
+            }
+            for (int c0 = 0; c0 < S; c0 += SS_STAGE) {
+                const int m = min(SS_STAGE, S - c0);
+                __syncthreads();
+                for (int j = tid; j < m; j += SS_T) U.sample[j] = R.k0[sample_place(c0 + j, stride)];
+                __syncthreads();
+                if (!act) continue;
+                // samples before the targets count if not larger, those after them if smaller
+                auto count = [&](int from, int to, int before) {   // before: 1, 0, or -1 for the targets' own 32
+                    for (int j = from + lane; j < to; j += 32) {
+                        const unsigned long long k = U.sample[j];
+#pragma unroll
+                        for (int u = 0; u < SS_TARGETS; u++) {
+                            const bool le = before < 0 ? c0 + j < i0 + u : before > 0;
+                            acc[u] += k < t[u] + (le ? 1 : 0);
+                        }
+                    }
+                };
+                const int own = i0 - c0;   // the targets' place in this chunk, if in it
+                const int e0 = min(m, max(0, own & ~31)), e1 = min(m, max(0, (own & ~31) + 32));
+                count(0, e0, 1);
+                count(e0, e1, -1);
+                count(e1, m, 0);
+            }
+#pragma unroll
+            for (int u = 0; u < SS_TARGETS; u++) {
+                const int rank = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(acc[u])));
+                if (act && lane == 0 && rank > 0 && rank % SS_OVER == 0) {
+                    A.scr->skey[rank / SS_OVER] = t[u];
+                    A.scr->spos[rank / SS_OVER] = static_cast<unsigned>(sample_place(i0 + u, stride));
+                }
+            }
+        }
+    }
+    if (!grid_sync(R.ctl, bar)) return;
+    // ---- 2. every key's bucket, and its place among the block's keys of it
+    int top = 1;
+    while (top < B) top <<= 1;
+    for (int i = tid; i < top; i += SS_T) {   // split[i]: the start of bucket i + 1
+        U.split.key[i] = i + 1 < B ? __ldcg(&A.scr->skey[i + 1]) : ~0ull;
+        U.split.pos[i] = i + 1 < B ? __ldcg(&A.scr->spos[i + 1]) : ~0u;
+    }
+    for (int i = tid; i < B; i += SS_T) U.split.cnt[i] = 0;
+    __syncthreads();
+    for (int i = b * SS_T + tid; i < n; i += G * SS_T) {
+        const unsigned long long k = R.k0[i];
+        int q = 0;
+        for (int step = top >> 1; step > 0; step >>= 1) {
+            const unsigned long long sk = U.split.key[q + step - 1];
+            if (sk < k || (sk == k && U.split.pos[q + step - 1] <= static_cast<unsigned>(i))) q += step;
+        }
+        R.v0[i] = static_cast<unsigned>(q) << 20 | static_cast<unsigned>(atomicAdd(&U.split.cnt[q], 1));
+    }
+    __syncthreads();
+    for (int i = tid; i < B; i += SS_T) {
+        const int c = U.split.cnt[i];
+        if (c) U.split.cnt[i] = atomicAdd(&A.scr->count[i], c);
+    }
+    if (!grid_sync(R.ctl, bar)) return;
+    // ---- 3. to the buckets
+    bool large = false;
+    {
+        int at = 0;
+        for (int i0 = 0; i0 < B; i0 += SS_T) {
+            const int c = i0 + tid < B ? __ldcg(&A.scr->count[i0 + tid]) : 0;
+            int total = 0;
+            const int x = block_excl_scan(c, s_warp, &total);
+            if (i0 + tid < B) s_start[i0 + tid] = at + x;
+            at += total;
+            large |= c > SS_CAP;
+        }
+        if (tid == 0) s_start[B] = at;
+    }
+    if (__syncthreads_or(large)) {   // the same in every block
+        for (int i = b * SS_T + tid; i < n; i += G * SS_T) R.v0[i] = static_cast<unsigned>(i);
+        if (!grid_sync(R.ctl, bar) || !radix_body(R, bar)) return;
+        if (A.order && grid_sync(R.ctl, bar))
+            for (int i = b * SS_T + tid; i < n; i += G * SS_T) A.order[i] = static_cast<long long>(__ldcg(&R.v0[i]));
+        return;
+    }
+    for (int i = b * SS_T + tid; i < n; i += G * SS_T) {
+        const unsigned e = R.v0[i], q = e >> 20;
+        const int at = s_start[q] + U.split.cnt[q] + static_cast<int>(e & 0xfffffu);
+        R.k1[at] = R.k0[i];
+        R.v1[at] = static_cast<unsigned>(i);
+    }
+    if (!grid_sync(R.ctl, bar)) return;
+    // ---- 4. the buckets sorted
+    for (int q = b; q < B; q += G) {
+        const int s0 = s_start[q], m = s_start[q + 1] - s0;
+        __syncthreads();
+        for (int i = tid; i < m; i += SS_T) {
+            U.bucket.key[i] = __ldcg(&R.k1[s0 + i]);
+            U.bucket.val[i] = __ldcg(&R.v1[s0 + i]);
+            U.bucket.claim[i] = 0;
+        }
+        __syncthreads();
+        for (bool again = false;; again = true) {
+            bool twice = false;
+            for (int i = tid; i < m; i += SS_T) {
+                const unsigned long long k = U.bucket.key[i];
+                const unsigned v = U.bucket.val[i];
+                int rank = 0;
+                if (!again) {
+#pragma unroll 8
+                    for (int j = 0; j < m; j++) rank += U.bucket.key[j] < k;
+                    twice |= atomicExch(&U.bucket.claim[rank], 1) != 0;
+                } else {
+                    for (int j = 0; j < m; j++) {
+                        const unsigned long long o = U.bucket.key[j];
+                        rank += o < k || (o == k && U.bucket.val[j] < v);
+                    }
+                }
+                R.k0[s0 + rank] = k;
+                if (A.order) A.order[s0 + rank] = static_cast<long long>(v);
+                else R.v0[s0 + rank] = v;
+            }
+            if (!__syncthreads_or(twice)) break;   // (never after the second ranking)
+        }
+    }
+}
+
+static SampleArgs sample_args(const RadixArgs &radix, SampleScratch *scr, long long *order = nullptr) {
+    SampleArgs A;
+    A.order = order;
+    A.radix = radix;
+    A.scr = scr;
+    A.buckets = sample_buckets(radix.n);
+    return A;
+}
+
+// The grid of a sample sort: a block per bucket or per 512 keys, to the cooperative limit.
+static int sample_grid(int n, int most) { return std::max(1, std::min(most, std::max(sample_buckets(n), (n + 511) / 512))); }
+
 // The epoch at which a context's sorts clear their status words: the constant
 // above, or a smaller value from NCORP_RADIX_EPOCH_LIMIT (read at context
 // creation; lets a test reach the clearing path in a few calls).
@@ -533,11 +766,12 @@ unsigned radix_epoch_limit() {
 }
 
 // Layout of the context's radix scratch (ints): two sets of digit histograms
-// of every pass at [0, 2 RS_MAX_PASSES 256), the epoch counter at RS_EPOCH_AT, the tile
-// status words from RS_STATUS_AT on.  The status words never share memory with anything
+// of every pass at [0, 2 RS_MAX_PASSES 256), the epoch counter at RS_EPOCH_AT, the sample
+// sort's buckets at RS_SAMPLE_AT, the tile status words from RS_STATUS_AT on.  The status words never share memory with anything
 // else, so a word left by an earlier sort (of any size) carries an older tag.
 constexpr int RS_EPOCH_AT = 2 * RS_MAX_PASSES * 256;
-constexpr int RS_STATUS_AT = 2 * RS_MAX_PASSES * 256 + 64;
+constexpr int RS_SAMPLE_AT = RS_EPOCH_AT + 64;
+constexpr int RS_STATUS_AT = RS_SAMPLE_AT + static_cast<int>(sizeof(SampleScratch) / sizeof(int));
 
 void ensure_radix_scratch(ncorp_ctx *c, int n) {
     const int ntiles = std::max(1, (n + RS_TILE - 1) / RS_TILE);
@@ -588,21 +822,35 @@ static RadixArgs radix_args(ncorp_ctx *c, uint64_t *keys, uint32_t *vals, uint64
     return A;
 }
 
-void radix_sort_u64(ncorp_ctx *c, uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, int n,
+// Sorts keys/vals in place (the alt buffers are scratch); the values are the
+// identity on entry; `bits` low bits of the key are significant (rounded up to
+// an even number of 8-bit passes, so the radix sort's result ends in the input
+// buffers).  bar_zeroed: the caller's stream has already zeroed ctl->bar_count
+// since the last cooperative kernel.  Up to SAMPLE_SORT_MAX keys of one disk take
+// the sample sort (which does not read the values), a forest's (disk, key) pairs and more keys the radix sort.
+void sort_u64(ncorp_ctx *c, uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, int n,
                     int bits, bool bar_zeroed, const int *gate, bool by_disk) {
     if (n <= 1) return;
     RadixArgs A = radix_args(c, keys, vals, keys_alt, vals_alt, n, bits, by_disk && c->nd > 1);
     A.gate = gate;
+    const bool sample = n <= SS_MAX_N && !(by_disk && c->nd > 1);
+    const void *kern = sample ? reinterpret_cast<const void *>(k_sample) : reinterpret_cast<const void *>(k_radix);
     int per_sm = 0;
-    NCORP_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reinterpret_cast<const void *>(k_radix),
-                                                                   RS_T, 0));
+    NCORP_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, RS_T, 0));
     if (per_sm < 1) per_sm = 1;
     if (per_sm > 2) per_sm = 2;
-    const int grid = std::min(A.ntiles, coop_blocks(c, per_sm));
     if (!bar_zeroed) NCORP_CUDA_CHECK(cudaMemsetAsync(&c->ctl->bar_count, 0, sizeof(unsigned), c->stream));
+    if (sample) {
+        SampleArgs SA = sample_args(A, reinterpret_cast<SampleScratch *>(c->tile_hist + RS_SAMPLE_AT));
+        void *args[] = {&SA};
+        NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(kern, dim3(sample_grid(n, coop_blocks(c, per_sm))), dim3(SS_T), args,
+                                                     0, c->stream));
+        c->launches++;
+        return;
+    }
+    const int grid = std::min(A.ntiles, coop_blocks(c, per_sm));
     void *args[] = {&A};
-    NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_radix), dim3(grid), dim3(RS_T), args,
-                                                 0, c->stream));
+    NCORP_CUDA_CHECK(cudaLaunchCooperativeKernel(kern, dim3(grid), dim3(RS_T), args, 0, c->stream));
     c->launches++;
 }
 
@@ -844,7 +1092,7 @@ __global__ void __launch_bounds__(RZ_T) k_resort(ResortArgs A) {
     if (b == 0 && t == 0) A.ctl->resort_ok = by_rank ? 1 : 2;
 }
 
-// Sorts keys (with idx = identity on entry) like radix_sort_u64 with the
+// Sorts keys (with idx = identity on entry) like sort_u64 with the
 // key bits of a Hilbert key, taking the fast path above when the keys are
 // nearly sorted.  ctl->bar_count must be zero on entry (k_keys zeroes it).
 void sort_near_sorted(ncorp_ctx *c, uint64_t *keys, uint32_t *idx, uint64_t *keys_alt, uint32_t *idx_alt, int n,
@@ -1006,12 +1254,15 @@ struct StaticScratch {
     unsigned long long status[256 * STATIC_TILES];
     int ghist[2 * RS_MAX_PASSES * 256];
     unsigned epoch;                   // radix sort calls so far (tags the status words)
+    SampleScratch sample;
 };
 
 static __device__ __align__(256) StaticScratch g_static_scratch;
 
+// One block.
 __global__ void k_static_reset(StaticScratch *S) {
-    for (int i = 0; i < 2 * RS_MAX_PASSES * 256; i++) S->ghist[i] = 0;
+    for (int i = threadIdx.x; i < 2 * RS_MAX_PASSES * 256; i += blockDim.x) S->ghist[i] = 0;
+    if (threadIdx.x) return;
     Ctrl &c = S->ctl;
     c.err = 0;
     c.bar_count = 0;
@@ -1026,23 +1277,25 @@ __global__ void k_static_reset(StaticScratch *S) {
     }
 }
 
-__global__ void k_static_split(const double *__restrict__ pos, StaticScratch *S, int n) {
+// The positions by component, and their box (see k_bbox).
+__global__ void __launch_bounds__(256) k_static_box(const double *__restrict__ pos, StaticScratch *S, int n) {
+    unsigned long long lo[3] = {~0ull, ~0ull, ~0ull}, hi[3] = {0ull, 0ull, 0ull};
+    bool bad = false;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        S->x[i] = pos[3 * i];
-        S->y[i] = pos[3 * i + 1];
-        S->z[i] = pos[3 * i + 2];
+        const double v[3] = {pos[3 * i], pos[3 * i + 1], pos[3 * i + 2]};
+        S->x[i] = v[0];
+        S->y[i] = v[1];
+        S->z[i] = v[2];
+#pragma unroll
+        for (int k = 0; k < 3; k++) fold_coordinate(v[k], lo[k], hi[k], bad);
     }
-}
-
-__global__ void k_static_order(const StaticScratch *S, int64_t *order, int n) {
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
-        order[i] = static_cast<int64_t>(S->idx[i]);
+    fold_box(lo, hi, bad, &S->ctl);
 }
 
 struct StaticDevice {
     StaticScratch *ptr = nullptr;
     int num_sms = 0;
-    int radix_per_sm = 0;
+    int sort_per_sm = 0;
 };
 
 static std::mutex g_static_mutex;
@@ -1060,10 +1313,10 @@ static cudaError_t static_setup(int dev, StaticDevice &out) {
         e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (e != cudaSuccess) return e;
         int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reinterpret_cast<const void *>(k_radix), RS_T, 0);
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, reinterpret_cast<const void *>(k_sample), SS_T, 0);
         if (e != cudaSuccess) return e;
         d.num_sms = sms;
-        d.radix_per_sm = std::max(1, std::min(per_sm, 2));
+        d.sort_per_sm = std::max(1, std::min(per_sm, 2));
         d.ptr = static_cast<StaticScratch *>(p);
     }
     out = d;
@@ -1103,18 +1356,16 @@ extern "C" int ncorp_hilbert_sort_static(const double *positions, int64_t n64, u
     {
         const int *no_gate = nullptr;
         void *a_reset[] = {&S};
-        void *a_split[] = {const_cast<double **>(&positions), &S, &ni};
-        void *a_bbox[] = {&sx, &sy, &sz, &ni, &ctl, &no_gate};
+        void *a_box[] = {const_cast<double **>(&positions), &S, &ni};
         void *a_keys[] = {&sx, &sy, &sz, &ni, &ctl, &keys, &sidx, &qx, &qy, &qz, &no_gate};
-        if (cudaLaunchKernel(reinterpret_cast<const void *>(k_static_reset), dim3(1), dim3(1), a_reset, 0, s) !=
+        if (cudaLaunchKernel(reinterpret_cast<const void *>(k_static_reset), dim3(1), dim3(512), a_reset, 0, s) !=
                 cudaSuccess ||
-            cudaLaunchKernel(reinterpret_cast<const void *>(k_static_split), dim3(g), dim3(256), a_split, 0, s) !=
+            cudaLaunchKernel(reinterpret_cast<const void *>(k_static_box), dim3(g), dim3(256), a_box, 0, s) !=
                 cudaSuccess ||
-            cudaLaunchKernel(reinterpret_cast<const void *>(k_bbox), dim3(g), dim3(256), a_bbox, 0, s) != cudaSuccess ||
             cudaLaunchKernel(reinterpret_cast<const void *>(k_keys), dim3(g), dim3(256), a_keys, 0, s) != cudaSuccess)
             return NCORP_ECUDA;
     }
-    if (n > 1) {
+    {
         RadixArgs A;
         A.k0 = keys; A.k1 = S->key_alt; A.v0 = S->idx; A.v1 = S->idx_alt;
         A.n = n;
@@ -1127,15 +1378,11 @@ extern "C" int ncorp_hilbert_sort_static(const double *positions, int64_t n64, u
         A.epoch_limit = RS_EPOCH_LIMIT;
         A.ctl = &S->ctl;
         A.gate = nullptr;
-        const int grid = std::min(A.ntiles, d.radix_per_sm * d.num_sms);
-        void *args[] = {&A};
-        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_radix), dim3(grid), dim3(RS_T), args, 0, s) !=
-            cudaSuccess)
-            return NCORP_ECUDA;
-    }
-    {
-        void *a_order[] = {&S, &order, &ni};
-        if (cudaLaunchKernel(reinterpret_cast<const void *>(k_static_order), dim3(g), dim3(256), a_order, 0, s) !=
+        static_assert(STATIC_MAX_N <= SS_MAX_N, "the sample sort takes every size");
+        SampleArgs SA = sample_args(A, &S->sample, reinterpret_cast<long long *>(order));
+        void *args[] = {&SA};
+        if (cudaLaunchCooperativeKernel(reinterpret_cast<const void *>(k_sample),
+                                        dim3(sample_grid(n, d.sort_per_sm * d.num_sms)), dim3(SS_T), args, 0, s) !=
             cudaSuccess)
             return NCORP_ECUDA;
     }
