@@ -21,6 +21,8 @@
 // leaf-leaf and leaf-self pieces covering exactly the same moonlet pairs (a
 // "forced" frontier entry that is only ever split), so that the direct lists
 // only hold leaves; the decision itself is counted once, where it is taken.
+#include <algorithm>
+
 #include "ctx.h"
 
 namespace ncorp {
@@ -745,8 +747,12 @@ void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     // (four blocks per SM take 300 us instead of 375 alone at N = 1e6, but in a step the launch waits for room
     // beside the multipoles: the step 2610 -> 2910 us)
     if (per_sm > 2) per_sm = 2;
-    // about one block per 640 moonlets (frontiers peak near a third of n pairs), 32 to the cooperative limit
-    const int grid = std::min(coop_blocks(c, per_sm), std::max(32, c->cur_n / 640));
+    // A block per 160 moonlets up to one per SM, then one per 640 up to the cooperative limit; at least 32.  Frontiers
+    // peak near a third of n pairs, several n with the smaller thresholds of low orders: the step with impacts at
+    // N = 3e4, p = 3 takes 591 us at 46 blocks and 505 at 188, the one at 5e4 405 (78) and 392 (304); with 304 blocks
+    // at N = 1e5 the launch waits for room beside the multipoles (541 us at 156, 556 at 304).
+    const int n = c->cur_n;
+    const int grid = std::min(coop_blocks(c, per_sm), std::max({32, std::min(n / 160, c->num_sms), n / 640}));
     if (gravity && collisions) k_walk_head<true, true><<<1, HEAD_THREADS, 0, c->stream>>>(A);
     else if (gravity) k_walk_head<true, false><<<1, HEAD_THREADS, 0, c->stream>>>(A);
     else k_walk_head<false, true><<<1, HEAD_THREADS, 0, c->stream>>>(A);
