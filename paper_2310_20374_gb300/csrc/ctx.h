@@ -131,6 +131,27 @@ __device__ __forceinline__ void walk_start(const WalkStart &W, Ctrl *ctl) {
 }
 #endif
 
+// What the host reads after a call, and where: the control blocks (and the error accumulator) in pinned host memory,
+// which the device writes directly (one copy per piece by the copy engine cost 17 us at the end of a step).
+struct Publish {
+    const Ctrl *ctl = nullptr, *ctl2 = nullptr;   // ctl2 null: the first alone
+    const int *acc = nullptr;
+    Ctrl *ctl_h = nullptr, *ctl2_h = nullptr;
+    int *acc_h = nullptr;
+};
+
+#ifdef __CUDACC__
+// by the threads of one block, after everything that writes the control blocks
+__device__ __forceinline__ void publish(const Publish &P) {
+    static_assert(sizeof(Ctrl) % sizeof(int) == 0, "copied by words");
+    for (int i = threadIdx.x; i < static_cast<int>(sizeof(Ctrl) / sizeof(int)); i += blockDim.x) {
+        reinterpret_cast<int *>(P.ctl_h)[i] = __ldcg(reinterpret_cast<const int *>(P.ctl) + i);
+        if (P.ctl2) reinterpret_cast<int *>(P.ctl2_h)[i] = __ldcg(reinterpret_cast<const int *>(P.ctl2) + i);
+    }
+    if (P.ctl2 && threadIdx.x == 0) *P.acc_h = __ldcg(P.acc);
+}
+#endif
+
 // Grid of a cooperative launch: the given blocks per SM, capped by the
 // context's limit so that the cooperative grids of contexts driven on
 // concurrent streams fit on the device together.
@@ -348,8 +369,10 @@ struct KickDriftArgs {
     float4 *cv4;
 };
 void launch_kick_drift(ncorp_ctx *c, const KickDriftArgs &A);
-void launch_scatter_state(ncorp_ctx *c, const ParticleSet &S, double *pos, double *vel, int n,
-                          const int *abort_a = nullptr, const int *abort_b = nullptr);
+// publishes P (the step's last kernel)
+void launch_scatter_state(ncorp_ctx *c, const ParticleSet &S, double *pos, double *vel, int n, const int *abort_a,
+                          const int *abort_b, const Publish &P);
+void launch_publish(ncorp_ctx *c, const Publish &P);
 void launch_unpack_pairs(ncorp_ctx *c, const uint64_t *packed, int64_t *out, int count);
 
 // host-side error helper used by every launcher

@@ -136,12 +136,13 @@ __global__ void __launch_bounds__(256) k_kick_drift(KickDriftArgs A) {
     if (threadIdx.x == 0 && s_bad) atomicOr(&A.ctl->err, ERR_NONFINITE);
 }
 
-// Positions and velocities to the caller's order in one pass.
+// Positions and velocities to the caller's order in one pass, and the control blocks to the host.
 __global__ void k_scatter_state(const double *__restrict__ x, const double *__restrict__ y,
                                 const double *__restrict__ z, const double *__restrict__ vx,
                                 const double *__restrict__ vy, const double *__restrict__ vz,
                                 const int *__restrict__ perm, double *__restrict__ pos, double *__restrict__ vel, int n,
-                                const int *abort_a, const int *abort_b) {
+                                const int *abort_a, const int *abort_b, const Publish P) {
+    if (blockIdx.x == 0) publish(P);
     if (scatter_gated(abort_a, abort_b)) return;
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         const int u = perm[i];
@@ -153,6 +154,8 @@ __global__ void k_scatter_state(const double *__restrict__ x, const double *__re
         vel[3 * u + 2] = vz[i];
     }
 }
+
+__global__ void k_publish(const Publish P) { publish(P); }
 
 static int eg(ncorp_ctx *c, int n) { return grid_for(n, 256, 16 * c->num_sms); }
 
@@ -174,12 +177,16 @@ void launch_kick_drift(ncorp_ctx *c, const KickDriftArgs &A) {
 }
 
 void launch_scatter_state(ncorp_ctx *c, const ParticleSet &S, double *pos, double *vel, int n, const int *abort_a,
-                          const int *abort_b) {
+                          const int *abort_b, const Publish &P) {
     k_scatter_state<<<eg(c, n), 256, 0, c->stream>>>(S.x, S.y, S.z, S.vx, S.vy, S.vz, S.perm, pos, vel, n, abort_a,
-                                                     abort_b);
+                                                     abort_b, P);
     c->launches++;
     NCORP_CUDA_CHECK(cudaGetLastError());
 }
 
+void launch_publish(ncorp_ctx *c, const Publish &P) {
+    k_publish<<<1, 128, 0, c->stream>>>(P); c->launches++;
+    NCORP_CUDA_CHECK(cudaGetLastError());
+}
 
 }  // namespace ncorp

@@ -532,14 +532,25 @@ void begin_call(ncorp_ctx *c) {
     }
 }
 
-// Waits for the call's work and returns its error word: the current tree
-// set's, and with both also the other set's and the accumulator's.
-int finish(ncorp_ctx *c, bool both = false) {
-    NCORP_CUDA_CHECK(cudaMemcpyAsync(c->ctl_h, c->ctl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
+// The current tree set's control block, and with both also the other set's and the error accumulator.
+Publish publication(const ncorp_ctx *c, bool both) {
+    Publish P;
+    P.ctl = c->ctl;
+    P.ctl_h = c->ctl_h;
     if (both) {
-        NCORP_CUDA_CHECK(cudaMemcpyAsync(c->alt.ctl_h, c->alt.ctl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
-        NCORP_CUDA_CHECK(cudaMemcpyAsync(c->err_acc_h, c->err_acc, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        P.ctl2 = c->alt.ctl;
+        P.ctl2_h = c->alt.ctl_h;
+        P.acc = c->err_acc;
+        P.acc_h = c->err_acc_h;
     }
+    return P;
+}
+
+// Waits for the call's work and returns its error word: the current tree
+// set's, and with both also the other set's and the accumulator's (published:
+// the work itself copied them to the host).
+int finish(ncorp_ctx *c, bool both = false, bool published = false) {
+    if (!published) launch_publish(c, publication(c, both));
     NCORP_CUDA_CHECK(cudaStreamSynchronize(c->stream));
     if (c->profile)
         for (int i = 0; i < NCORP_NSTAGES; i++) {
@@ -713,7 +724,7 @@ void collisions_standard(ncorp_ctx *c, const ParticleSet &S, int n, double dt) {
 // tree sets have traded places (the current one describes the new positions)
 // and the new state is in Cset (not yet swapped with A); nothing is copied to
 // the caller and nothing waits: the caller reads the status.
-void enqueue_kdk(ncorp_ctx *c, int n, int p, double theta, double dt, bool overlap) {
+void enqueue_kdk(ncorp_ctx *c, int n, int p, double theta, double dt, bool overlap, bool fresh = false) {
     const double h = 0.5 * dt;
     ParticleSet &A = c->A, &B = c->B, &Cn = c->Cset;
     const bool resolve = c->cfg.collisions && c->cfg.resolve_f > 0.0;
@@ -724,8 +735,9 @@ void enqueue_kdk(ncorp_ctx *c, int n, int p, double theta, double dt, bool overl
     // the other tree set becomes the new tree's: cleared (its errors kept) before the kick-drift
     // kernel folds the drifted positions' bounding box into its control block.  It also takes over
     // the abort bits of A's tree: if A's acceleration was never computed (an overflow in the same
-    // call), the kick-drift and everything built from it do nothing.
-    on_alt(c, [&] { reset_ctl(c, true); });
+    // call), the kick-drift and everything built from it do nothing.  (fresh:
+    // both sets were just cleared and nothing has run on them since.)
+    if (!fresh) on_alt(c, [&] { reset_ctl(c, true); });
     {
         Stage st(c, NCORP_STAGE_KDK);
         KickDriftArgs K;
@@ -878,11 +890,12 @@ void drop_graph(StepGraph &g) {
 void resident_step_body(ncorp_ctx *c, double *pos, double *vel, int n, int p, double theta, double dt, bool dev_x,
                         bool dev_v) {
     reset_ctls(c);
-    enqueue_kdk(c, n, p, theta, dt, true);
+    enqueue_kdk(c, n, p, theta, dt, true, true);
     Stage st(c, NCORP_STAGE_KDK);
     ParticleSet &Cn = c->Cset;
     // a step that aborted (overflow, time-out) writes nothing to the caller's arrays
-    launch_scatter_state(c, Cn, dev_x ? pos : c->stage, dev_v ? vel : c->stage2, n, &c->ctl->err, &c->alt.ctl->err);
+    launch_scatter_state(c, Cn, dev_x ? pos : c->stage, dev_v ? vel : c->stage2, n, &c->ctl->err, &c->alt.ctl->err,
+                         publication(c, true));
 }
 
 // Enqueues a resident step on c->stream through a cached graph (capturing it
@@ -1312,7 +1325,7 @@ int ncorp_step(ncorp_ctx *c, double *positions, double *velocities, const double
                 download_vec(c, Cn.vx, Cn.vy, Cn.vz, Cn.perm, velocities, n, c->stage2, &c->ctl->err,
                              &c->alt.ctl->err);
             }
-            const int err = finish(c, true);
+            const int err = finish(c, true, c->graph_used);
             // the current tree set now holds the new tree, the other one A's tree
             const int e_new = c->ctl_h->err, e_old = c->alt.ctl_h->err, e_acc = *c->err_acc_h;
             if (err & ERR_NONFINITE) {
@@ -2352,9 +2365,7 @@ int ncorp_batch_run(ncorp_batch *b, int n_steps) {
             begin_call(c);
             choose_parameters(c, f->p);
             enqueue_run(*f, n_steps);
-            NCORP_CUDA_CHECK(cudaMemcpyAsync(c->ctl_h, c->ctl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
-            NCORP_CUDA_CHECK(cudaMemcpyAsync(c->alt.ctl_h, c->alt.ctl, sizeof(Ctrl), cudaMemcpyDeviceToHost, c->stream));
-            NCORP_CUDA_CHECK(cudaMemcpyAsync(c->err_acc_h, c->err_acc, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+            launch_publish(c, publication(c, true));
         }
         for (int s = 0; s < BATCH_STREAMS; s++) {
             NCORP_CUDA_CHECK(cudaEventRecord(b->ev_done[s], b->pool[s]));
