@@ -88,7 +88,17 @@ constexpr int WALK_MAX_ITERS = 96;
 // G = floor(32 / ceil(m / 2)) groups, so 33 to 52 targets (one group, 52 to 81 %
 // of the lanes) go better as 32 (two groups, every lane) and the rest, although
 // the sources are then staged twice.
-__host__ __device__ inline int near_targets(int m) { return m > 64 ? 64 : (m > 32 && m <= 52 ? 32 : m); }
+// The FP64 kernel takes all of a leaf's entries and few targets: its lanes hold the sources, which few entries
+// would not fill, and a warp instruction takes so long that an item must be few of them.
+constexpr int NEAR64_TARGETS = 16;   // (64 in leaves of more than 256, to bound the items)
+__host__ __device__ inline int near_targets(int m, bool fp64) {
+    if (m > (fp64 ? 256 : 64)) return 64;
+    if (fp64) {
+        const int parts = (m + NEAR64_TARGETS - 1) / NEAR64_TARGETS;
+        return (m + parts - 1) / parts;
+    }
+    return m > 32 && m <= 52 ? 32 : m;
+}
 
 // Equal shares of E direct entries for m targets: NEAR_ENTRIES G source leaves
 // of some sixteen moonlets each are about forty rounds of the kernel's loop
@@ -96,7 +106,11 @@ __host__ __device__ inline int near_targets(int m) { return m > 64 ? 64 : (m > 3
 // items per warp of the device, down to four entries (an item's fixed cost is
 // about that of four).
 constexpr int NEAR_ENTRIES = 10, NEAR_ENTRIES_MIN = 4, NEAR_ITEMS_WANTED = 8192;
-__host__ __device__ inline int near_shares(int E, int m, int n_leaves) {
+__host__ __device__ inline int near_shares(int E, int m, int n_leaves, bool fp64) {
+    if (fp64) {   // 12 to 96 entries, by the leaves: 425 to 407 us a step at N = 1e4 (48: 504), 5160 to 4130 at 1e5 (32: 4250)
+        const int per = n_leaves / 48 < 12 ? 12 : (n_leaves / 48 > 96 ? 96 : n_leaves / 48);
+        return (E + per - 1) / per;
+    }
     long long e = NEAR_ENTRIES * (32 / ((m + 1) / 2));
     if (n_leaves < NEAR_ITEMS_WANTED) e = e * n_leaves / NEAR_ITEMS_WANTED;
     const int per = e < NEAR_ENTRIES_MIN ? NEAR_ENTRIES_MIN : static_cast<int>(e);

@@ -144,4 +144,27 @@ __device__ __forceinline__ void p2p_f64(double jx, double jy, double jz, double 
     az += dz * f3;
 }
 
+// mu / r^3 of one near-field pair for both moonlets, FP64: fj = mj r^-3 and
+// fi = mi r^-3 from r^2, 8 FP64 instructions (a divide and a square root
+// alone take 18), in the way of p2p_f64.
+__device__ __forceinline__ void p2p_f64_both(double r2, double mj, double mi, double &fj, double &fi) {
+    const unsigned hi = static_cast<unsigned>(__double2hiint(r2)), lo = static_cast<unsigned>(__double2loint(r2));
+    if ((hi >> 20) - (1023u - 120u) <= 240u) {
+        const unsigned yb = __float_as_uint(rsqrtf(__uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29))));
+        const double y = __hiloint2double(static_cast<int>((yb >> 3) + (896u << 20)), static_cast<int>(yb << 29));
+        const double y2 = y * y;
+        const double e = fma(-r2, y2, 1.0);
+        const double c = e * fma(e, 1.875, 1.5);
+        const double g = y * y2, f = fma(g, c, g);
+        fj = mj * f;
+        fi = mi * f;
+    } else if (r2 > 0.0) {
+        const double inv = 1.0 / sqrt(r2);
+        fj = mj * inv * inv * inv;
+        fi = mi * inv * inv * inv;
+    } else {
+        fj = fi = 0.0;
+    }
+}
+
 }  // namespace ncorp

@@ -38,8 +38,9 @@ struct NearWindow {
     int first, before;   // this lane's entry
     int total;           // moonlets of the window
     __device__ __forceinline__ void load(const int2 *src, int at, int end, int lane) {
-        int2 e = make_int2(0, 0);
-        if (at + lane < end) e = __ldg(&src[at + lane]);
+        set(at + lane < end ? __ldg(&src[at + lane]) : make_int2(0, 0), lane);
+    }
+    __device__ __forceinline__ void set(int2 e, int lane) {
         int incl = e.y;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
@@ -313,79 +314,103 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {
 }
 
 // FP64: bound by the FP64 pipe (one warp instruction per 64 cycles per SM
-// sub-partition).  p2p_f64 takes 16 FP64 instructions a pair where the divide
-// and square root of the plain form took about 29.  One block per leaf and
-// share of its direct list, the targets in G = floor(NEAR_THREADS / m) groups:
-// the pipe is the limit, so every lane counts (97 % of them work at 25 targets
-// a leaf, 78 % with a warp per leaf and a target per lane).  N = 1e5, p = 6: 7.9
-// -> 3.6 ms.
-constexpr int NEAR_BUF = 256;   // sources a block stages at a time
+// sub-partition), so a pair of leaves is summed once for both: the separation
+// and r^-3 serve the pull on either moonlet, 20 FP64 instructions for what
+// takes 32 as two pulls.  Of an item's entries those with a later leaf count
+// (and the leaf itself, one way).  A block takes an item, each warp a quarter
+// of its targets (a pair of leaves keeps one warp's share of the pipe busy for
+// half a millisecond) and all its sources, 32 at a time, one per lane, so that all
+// lanes work whatever the leaves' sizes.  A warp goes through its m targets with
+// lane l starting at target l mod m: the lanes' pulls on the targets go to distinct places of the warp's
+// sums in shared memory (lanes that would meet have copies of the sums), those on the lane's source stay in registers.  Both are added to the
+// moonlets' sums in memory with FP64 atomics.  N = 1e5, p = 6, beside M2L:
+// 3.57 ms one way (a block per leaf and share, 97 % of the lanes at work), 2.6 ms
+// this way; both near their instructions' time.  With a warp's items cut by
+// entries instead (few sources, many targets) 3.2 ms, and at N = 1e4 twice the one-way time.
+constexpr int NEAR64_SHARE = 64 / NEAR_WARPS, NEAR64_SUMS = 3 * NEAR64_SHARE;   // targets and sums of a warp
 
-struct __align__(16) NearShared64 {
-    double s[4][NEAR_BUF];           // x, y, z, mu of the staged sources
-    double red[3][NEAR_THREADS];
-    int item;
+struct __align__(16) NearShared64 {             // of a warp
+    double t[4][NEAR64_SHARE];                  // x, y, z, mu of its targets
+    double sum[3][NEAR64_SUMS];                 // pulls on them: copies of m sums
 };
 
 __global__ void __launch_bounds__(NEAR_THREADS, 6) k_near_f64(NearArgs A) {
-    __shared__ NearShared64 S;
+    __shared__ NearShared64 s_warp[NEAR_WARPS];
+    __shared__ int s_item[2];
     if (aborted(A.ctl)) return;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    NearShared64 &S = s_warp[warp];
     const int n_items = min(A.ctl->n_near, A.item_cap);
-    while (true) {
-        __syncthreads();   // every thread has read S.item
-        if (tid == 0) S.item = atomicAdd(A.work, 1);
-        __syncthreads();
-        const int li = S.item;
+    for (int turn = 0;; turn ^= 1) {
+        if (threadIdx.x == 0) s_item[turn] = atomicAdd(A.work, 1);
+        __syncthreads();   // (the item before last, of this slot, has been read by every thread)
+        const int li = s_item[turn];
         if (li >= n_items) break;
         const NearItem I(__ldg(&A.items[li]));
-        const int m = I.count;   // at most 64
-        const int G = NEAR_THREADS / m, g = tid / m, tt = tid - g * m;
-        const bool act = g < G;
-        const int i = I.first + (act ? tt : 0);
-        const double X = A.x[i], Y = A.y[i], Z = A.z[i];
-        double ax = 0.0, ay = 0.0, az = 0.0;
+        // the warp's share of the item's targets (at most 64)
+        const int first = I.first + I.count * warp / NEAR_WARPS, m = I.first + I.count * (warp + 1) / NEAR_WARPS - first;
+        if (m == 0) continue;
+        if (lane < m) {
+            S.t[0][lane] = A.x[first + lane];
+            S.t[1][lane] = A.y[first + lane];
+            S.t[2][lane] = A.z[first + lane];
+            S.t[3][lane] = A.G * A.m[first + lane];
+        }
+#pragma unroll
+        for (int d = 0; d < 3; d++) S.sum[d][lane] = S.sum[d][16 + lane] = 0.0;
+        const int copy = lane / m, i_first = lane - copy * m;   // (32 lanes, m <= 16: places 0 to 31, the last copy cut)
+        __syncwarp();
         NearWindow W;
         for (int at = I.s0; at < I.s1; at += 32) {
-            W.load(A.p2p_src, at, I.s1, lane);
-            for (int pos = 0; pos < W.total; pos += NEAR_BUF) {
-                const int total = min(NEAR_BUF, W.total - pos);
-                __syncthreads();
+            // the window's entries: later leaves, and the targets' own
+            int2 e = make_int2(0, 0);
+            if (at + lane < I.s1) e = __ldg(&A.p2p_src[at + lane]);
+            const bool own = e.x <= I.first && I.first < e.x + e.y;
+            const unsigned which = __ballot_sync(0xffffffffu, own);
+            const int o0 = __shfl_sync(0xffffffffu, e.x, __ffs(which) - 1), o1 = o0 + __shfl_sync(0xffffffffu, e.y, __ffs(which) - 1);
+            const unsigned keep = __ballot_sync(0xffffffffu, e.y > 0 && (own || e.x > I.first));
+            const unsigned from = __fns(keep, 0, lane + 1);   // (a window's entries are not empty)
+            e.x = __shfl_sync(0xffffffffu, e.x, from & 31);
+            e.y = __shfl_sync(0xffffffffu, e.y, from & 31);
+            W.set(from < 32 ? e : make_int2(0, 0), lane);
+            for (int pos = 0; pos < W.total; pos += 32) {
+                const int j = W.moonlet(pos, lane);
+                const bool valid = j >= 0, both = valid && !(which && j >= o0 && j < o1);
+                double X = 0.0, Y = 0.0, Z = 0.0, M = 0.0, ax = 0.0, ay = 0.0, az = 0.0;
+                if (valid) {
+                    X = A.x[j];
+                    Y = A.y[j];
+                    Z = A.z[j];
+                    M = A.G * A.m[j];
+                }
+                for (int s = 0, i = i_first; s < m; s++) {
+                    const int q = copy * m + i;
+                    const double mu = S.t[3][i];
+                    const double dx = X - S.t[0][i], dy = Y - S.t[1][i], dz = Z - S.t[2][i];
+                    double fi, fj;   // mu r^-3 of the source's pull on the target and of the target's on the source
+                    p2p_f64_both(dx * dx + dy * dy + dz * dz, M, mu, fi, fj);
+                    if (!valid) fi = 0.0;   // (a lane past the sources)
+                    const double sx = S.sum[0][q], sy = S.sum[1][q], sz = S.sum[2][q];
+                    S.sum[0][q] = sx + dx * fi;
+                    S.sum[1][q] = sy + dy * fi;
+                    S.sum[2][q] = sz + dz * fi;
+                    ax -= dx * fj;
+                    ay -= dy * fj;
+                    az -= dz * fj;
+                    i = i + 1 < m ? i + 1 : 0;
+                    __syncwarp();   // the next lane's turn at this target
+                }
+                if (both) near_store(A, j, false, ax, ay, az);
+            }
+        }
+        if (lane < m) {   // the copies of the sums
+            double v[3] = {0.0, 0.0, 0.0};
+            for (int q = lane; q < NEAR64_SUMS; q += m)
 #pragma unroll
-                for (int r = 0; r < NEAR_BUF / NEAR_THREADS; r++) {
-                    const int t0w = 32 * (warp + NEAR_WARPS * r), t = t0w + lane;
-                    const int j = W.moonlet(pos + t0w, lane);
-                    if (j >= 0) {
-                        S.s[0][t] = A.x[j];
-                        S.s[1][t] = A.y[j];
-                        S.s[2][t] = A.z[j];
-                        S.s[3][t] = A.G * A.m[j];
-                    }
-                }
-                __syncthreads();
-                if (act) {
-#pragma unroll 2
-                    for (int k = g; k < total; k += G)
-                        p2p_f64(S.s[0][k], S.s[1][k], S.s[2][k], S.s[3][k], X, Y, Z, ax, ay, az);
-                }
-            }
+                for (int d = 0; d < 3; d++) v[d] += S.sum[d][q];
+            near_store(A, first + lane, false, v[0], v[1], v[2]);
         }
-        if (G > 1) {
-            __syncthreads();
-            S.red[0][tid] = ax;
-            S.red[1][tid] = ay;
-            S.red[2][tid] = az;
-            __syncthreads();
-            if (g == 0) {
-                ax = ay = az = 0.0;
-                for (int q = 0; q < G; q++) {
-                    ax += S.red[0][q * m + tt];
-                    ay += S.red[1][q * m + tt];
-                    az += S.red[2][q * m + tt];
-                }
-            }
-        }
-        if (g == 0 && act) near_store(A, i, I.whole, ax, ay, az);
+        __syncwarp();   // the sums have been read
     }
 }
 

@@ -57,6 +57,7 @@ struct WalkArgs {
     int2 *p2p_src;             // per directed near-field entry: the source leaf's (first, count)
     int4 *near_items;          // near-field work items (count ctl->n_near)
     int near_cap;
+    bool fp64;                 // the FP64 near field follows
     const int *first;
     int2 *m2l_dir;
     int m2l_dir_cap, p2p_dir_cap;
@@ -180,7 +181,7 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
             // the near field's items: a subset of the leaf's moonlets and an equal share of its entries each
             const int m = vp > 0 ? __ldg(&A.count[i]) : 0;
             int parts = 0;
-            for (int t = 0; t < m; t += near_targets(m - t)) parts += near_shares(vp, near_targets(m - t), n_leaves);
+            for (int t = 0; t < m; t += near_targets(m - t, A.fp64)) parts += near_shares(vp, near_targets(m - t, A.fp64), n_leaves, A.fp64);
             int total_items = 0;
             const int xi = block_prefix(parts, s_tmp, &total_items);
             if (threadIdx.x == 0) s_items = total_items ? atomicAdd(&A.ctl->n_near, total_items) : 0;
@@ -191,8 +192,8 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
                 if (slot + parts > A.near_cap || s0 + vp > A.p2p_dir_cap) {
                     atomicOr(&A.ctl->err, ERR_DIRECTED);
                 } else {
-                    for (int t = 0; t < m; t += near_targets(m - t)) {
-                        const int k = near_targets(m - t), np = near_shares(vp, k, n_leaves);
+                    for (int t = 0; t < m; t += near_targets(m - t, A.fp64)) {
+                        const int k = near_targets(m - t, A.fp64), np = near_shares(vp, k, n_leaves, A.fp64);
                         for (int q = 0; q < np; q++)
                             A.near_items[slot++] = make_int4(f + t, np == 1 ? k : -k,
                                                              s0 + static_cast<int>(static_cast<long long>(vp) * q / np),
@@ -735,7 +736,7 @@ void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     A.cp2p = W.cp2p; A.cp2p_cap = W.p2p_cap;
     A.cself = W.cself; A.cself_cap = W.self_cap;
     A.cnt = W.cnt; A.offs = W.offs; A.cursor = W.cursor; A.p2p_off = W.p2p_off; A.p2p_src = W.p2p_src;
-    A.near_items = W.near_items; A.near_cap = W.near_cap;
+    A.near_items = W.near_items; A.near_cap = W.near_cap; A.fp64 = !c->grav_mixed;
     A.m2l_dir = W.m2l_dir; A.m2l_dir_cap = W.m2l_dir_cap; A.p2p_dir_cap = W.p2p_dir_cap;
     A.ctl = c->ctl;
     const void *kern = gravity && collisions ? reinterpret_cast<const void *>(k_walk<true, true>)

@@ -46,3 +46,24 @@ def test_direct_sum(n, leaf, fp64):
     tol = 40 * 2.0 ** -24 + 3 * 2.0 ** -48 * 16 / 1e-7 if not fp64 else (n + 40) * 2.0 ** -53
     err = np.linalg.norm(mut - ref, axis=1)
     assert np.all(err <= tol * scale), float(np.max(err / np.maximum(scale, 1e-300)))
+
+
+@pytest.mark.parametrize("n,leaf", [(1500, 3), (1500, 40), (1500, 64), (1500, 260), (4003, 17), (4003, 700)])
+def test_fp64_pairs_serve_both_moonlets(n, leaf):
+    """Several leaves and several items a leaf: every pair pulls on both moonlets once (the sum of forces is zero)."""
+    import torch
+    from paper_2310_20374_gb300 import ncorp
+    d = diskgen.make_disk(n, 17 + leaf)
+    pos, m = d["pos"].copy(), d["mass"]
+    cfg = ncorp.ncorp_config_default()
+    cfg.precision, cfg.leaf_size = ncorp.NCORP_FP64, leaf
+    cfg.n_cs = cfg.n_cc_pre = cfg.n_cc_post = 1 << 30
+    ctx = ncorp.ncorp_init(cfg, n, 0, torch.cuda.current_stream().cuda_stream)
+    try:
+        acc, mut = np.zeros((n, 3)), np.zeros((n, 3))
+        ncorp.ncorp_accel(ctx, pos, m, n, 3, 0.5, acc, mut)
+    finally:
+        ncorp.ncorp_free(ctx)
+    ref, scale = direct(pos, m)
+    assert np.all(np.linalg.norm(mut - ref, axis=1) <= (n + 40) * 2.0 ** -53 * scale)
+    assert np.all(np.abs((m[:, None] * mut).sum(0)) <= (n + 40) * 2.0 ** -53 * (m * scale).sum())
