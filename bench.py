@@ -35,12 +35,10 @@ if ROOT not in sys.path:
 
 METRIC = "particle-steps/s, falcON p=6 gravity+collisions; p50/p99 step latency mixed-N"
 UNIT = "particle-steps/s"
-# DRAM bytes (read + write) of one k_eval launch, from ncu captures of the current
+# DRAM bytes (read + write) of one near-field launch, from ncu captures of the current
 # kernel (dram__bytes_read.sum + dram__bytes_write.sum, mixed precision, leaf size
 # 64), keyed by (N, p, theta_min); entries are removed whenever the kernel changes,
-# until it is captured again.  Other workloads report null.  Empty: the captures
-# (5.54e6 at N = 1e5, p = 6; 50.3e6 at N = 1e6, p = 4) were taken with the kernel
-# at eight blocks per SM, before its launch bound became six.
+# until it is captured again.  Other workloads report null.
 EVAL_DRAM_BYTES_PER_LAUNCH = {}
 
 
@@ -381,14 +379,14 @@ def time_disk(a, ncorp, torch, ctx_args, d, n, p, theta, precision, steps, warmu
 
 
 def near_roofline(t, peak_tflops, precision, traffic):
-    """Roofline of the dominant kernel, the near-field direct sums (k_eval): NEAR_FLOP_PER_PAIR per unordered
+    """Roofline of the dominant kernel, the near-field direct sums (k_near_f32 or k_near_f64): NEAR_FLOP_PER_PAIR per unordered
     moonlet pair of the step (the method's count, whatever the kernel evaluates) over the kernel's event-timed
     duration, against the measured FMA peak of its precision."""
     near_ms = t["stage"].get("near", 0.0)
     pairs = t["prof"]["p2p_interactions"]
     flops = NEAR_FLOP_PER_PAIR * pairs
     achieved = flops / (near_ms * 1e-3) / 1e12 if near_ms > 0 else 0.0
-    return {"bound": "alu", "kernel": "k_eval (near-field direct sums per leaf)",
+    return {"bound": "alu", "kernel": f"k_near_{'f32' if precision == 'mixed' else 'f64'} (near-field direct sums per leaf)",
             "achieved": round(achieved, 3), "peak": round(peak_tflops, 2), "unit": "TFLOP/s",
             "frac": round(achieved / peak_tflops, 4) if peak_tflops else None, "traffic": traffic,
             "flops_per_launch": flops, "unordered_pairs_per_launch": pairs, "avg_launch_ms": round(near_ms, 4),
