@@ -82,10 +82,13 @@ __device__ __forceinline__ void test_and_emit(const CollideArgs &A, int u, int v
 //  2. The trajectories come within R1 + R2 of each other at the impact time
 //     dt_c in [0, dt], so the least distance over [0, dt] is at most R1 + R2:
 //     with t* = clamp(-dr.dv / dv^2, 0, dt), |dr + t* dv|^2 against
-//     (R1 + R2)^2 (1 + 2^-10) plus 2^-12 (|dr|^2 + dt^2 |dv|^2).  The margin
-//     exceeds the FP32 evaluation's error (velocities rounded to FP32: ~1e-7
-//     relative; the terms of the quadratic are bounded by that scale) by
-//     orders of magnitude, and the FP64 predicate's rounding likewise.
+//     (R1 + R2)^2 (1 + 2^-9) plus 2^-12 (|dr|^2 + dt^2 |dv|^2) plus 1025
+//     delta^2.  delta = dt 2^-23 (|v1| + |v2|, sums of components) is what the velocities'
+//     rounding to FP32 can move a trajectory by, so also the least distance (where |dv| is
+//     below the velocities' FP32 resolution it is all that dv says):
+//     (Rs + delta)^2 <= Rs^2 (1 + 2^-10) + 1025 delta^2.  The margin
+//     exceeds the FP32 evaluation's error (the terms of the quadratic are bounded by that
+//     scale) by orders of magnitude, and the FP64 predicate's rounding likewise.
 __device__ __forceinline__ bool may_touch(const float4 &h, const float4 &l, float r, const float4 &th,
                                           const float4 &tl, float tr, float &dx, float &dy, float &dz) {
     dx = (h.x - th.x) + (l.x - tl.x);
@@ -103,8 +106,9 @@ __device__ __forceinline__ bool may_meet(float dx, float dy, float dz, const flo
     const float t = u2 > 0.0f ? fminf(fmaxf(-b / u2, 0.0f), dt) : 0.0f;
     const float ex = dx + t * ux, ey = dy + t * uy, ez = dz + t * uz;
     const float d2 = dx * dx + dy * dy + dz * dz;
-    const float margin = 0x1p-12f * (d2 + dt * dt * u2) + 1e-30f;
-    return ex * ex + ey * ey + ez * ez <= Rs * Rs * (1.0f + 0x1p-10f) + margin;
+    const float dl = dt * 0x1p-23f * (fabsf(v.x) + fabsf(v.y) + fabsf(v.z) + fabsf(tv.x) + fabsf(tv.y) + fabsf(tv.z));
+    const float margin = 0x1p-12f * (d2 + dt * dt * u2) + 1025.0f * dl * dl + 1e-30f;
+    return ex * ex + ey * ey + ez * ez <= Rs * Rs * (1.0f + 0x1p-9f) + margin;
 }
 
 constexpr int COL_WARPS = 8;
