@@ -111,6 +111,27 @@ __device__ __forceinline__ bool may_meet(float dx, float dy, float dz, const flo
     return ex * ex + ey * ey + ez * ez <= Rs * Rs * (1.0f + 0x1p-9f) + margin;
 }
 
+// A pair that overlaps already cannot collide: with dr^2 < (R1 + R2)^2 Delta exceeds (dr.dv)^2, so dt_c < 0.  In FP32
+// with a margin of 2^-7 on the squares (both are good to 2^-18), where Delta exceeds (dr.dv)^2 by 2^-7 of itself and
+// the FP64 test's rounding cannot turn the sign; not where the separation or dv is near the resolution of the
+// positions' FP32 pairs (s: a bound on the position's size) or the squares near FP32's range.  In a dense ring most pairs
+// that pass test 2 overlap, and each sent its warp through some 3000 cycles of the FP64 pipe (60 % busy): with this and
+// radius_f32 the kernel alone goes from 275 to 148 us on a ring of N = 2e5, from 100 to 48 in the step with impacts at 3e4.
+__device__ __forceinline__ bool overlapping(float dx, float dy, float dz, const float4 &v, const float4 &tv, float Rs,
+                                            float s) {
+    const float ux = v.x - tv.x, uy = v.y - tv.y, uz = v.z - tv.z;
+    const float d2 = dx * dx + dy * dy + dz * dz, u2 = ux * ux + uy * uy + uz * uz, R2 = Rs * Rs;
+    return d2 < R2 * (1.0f - 0x1p-7f) && R2 > 1e-24f && R2 < 1e30f && Rs > 0x1p-30f * s && u2 > 1e-20f;
+}
+
+// A radius in FP32, at most 2^-23 of it below: cut by integer instructions (a conversion takes the FP64 pipe; three of
+// them per item were a fifth of its time).
+__device__ __forceinline__ float radius_f32(double R) {
+    const unsigned hi = static_cast<unsigned>(__double2hiint(R)), lo = static_cast<unsigned>(__double2loint(R));
+    if ((hi >> 20) - 897u < 254u) return __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
+    return static_cast<float>(R);   // zero, or outside FP32's normal range
+}
+
 constexpr int COL_WARPS = 8;
 
 // 3. Before the pairs of two different leaves A and B are formed, each
@@ -187,7 +208,7 @@ __global__ void __launch_bounds__(32 * COL_WARPS, 4) k_collide(CollideArgs A) {
                 th = A.hi4[ft + u];
                 tl = A.lo4[ft + u];
                 tv = A.cv[ft + u];
-                tR = static_cast<float>(A.R[ft + u]);
+                tR = radius_f32(A.R[ft + u]);
             }
             for (int j0 = 0; j0 < nsrc; j0 += COL_STAGE) {
                 const int lim = min(COL_STAGE, nsrc - j0);
@@ -210,7 +231,7 @@ __global__ void __launch_bounds__(32 * COL_WARPS, 4) k_collide(CollideArgs A) {
                         s_h[wl][slot] = h;
                         s_l[wl][slot] = l;
                         s_v[wl][slot] = v;
-                        s_R[wl][slot] = static_cast<float>(A.R[fs + j0 + k]);
+                        s_R[wl][slot] = radius_f32(A.R[fs + j0 + k]);
                         s_j[wl][slot] = j0 + k;
                     }
                     cnt += __popc(bal);
@@ -221,7 +242,8 @@ __global__ void __launch_bounds__(32 * COL_WARPS, 4) k_collide(CollideArgs A) {
                         const int v = s_j[wl][k];
                         float dx, dy, dz;
                         if ((!self || v > u) && may_touch(s_h[wl][k], s_l[wl][k], s_v[wl][k].w, th, tl, tv.w, dx, dy, dz) &&
-                            may_meet(dx, dy, dz, s_v[wl][k], tv, (s_R[wl][k] + tR) * (1.0f + 0x1p-20f), dtf))
+                            may_meet(dx, dy, dz, s_v[wl][k], tv, (s_R[wl][k] + tR) * (1.0f + 0x1p-20f), dtf) &&
+                            !overlapping(dx, dy, dz, s_v[wl][k], tv, s_R[wl][k] + tR, fabsf(th.x) + fabsf(th.y) + fabsf(th.z)))
                             test_and_emit(A, ft + u, fs + v);
                     }
                 }
