@@ -109,7 +109,7 @@ struct Ctrl {
                            // of the same tree set)
     unsigned bar_build;    // the build's grid barrier
     unsigned bar_walk;     // the walk's grid barrier
-    int walk_head;         // generation the walk's first block left to all of them (-1: a list was full)
+    int walk_head;         // generation the walk's head left to all the blocks (-1: none, nothing to walk)
     int walk_abort[3];     // walk: overflow seen in generation g, slot g mod 3
     long long dec_pairs;   // walk decisions: direct cell pairs
     long long dec_self;    // walk decisions: direct self cells

@@ -38,7 +38,7 @@ struct WalkArgs {
     int gravity;               // the gravity criterion is walked (its lists, per-target lists, statistics)
     int collisions;            // the collision criterion is walked (pairs into cp2p / cself)
     WalkCrit g, c;             // gravity and collision criteria
-    const int *gate;           // nullable: the walk does nothing while *gate is 0
+    const int *gate;           // nullable: the walk does nothing while *gate is 0 (read by the head)
     int2 *cp2p;                // collision walk: leaf pairs to test (count ctl->n_cp2p)
     int *cself;                // collision walk: leaves to test within (count ctl->n_cself)
     int cp2p_cap, cself_cap;
@@ -496,7 +496,8 @@ __device__ __forceinline__ bool walk_emit(const WalkArgs &A, const WalkOut &o, c
 // memory, the reservations' atomics and the grid barrier make it 4 us, and
 // the first five generations of a large tree hold a few hundred pairs.  Leaves
 // the next generation's pairs in the frontier buffer and its number in
-// ctl->walk_head (-1: a list was full).  A launch of its own: with the head's
+// ctl->walk_head (-1: the walk ends here, because a list was full, an earlier stage
+// failed or the gate is closed).  A launch of its own: with the head's
 // shared memory in every block of the walk, the SMs would not take the walk's blocks
 // beside those of the kernels on the other streams (150 us of the step at N = 1e6).
 // Head and walk in the step at N = 1e5, with the resets moved into the climb and
@@ -536,9 +537,12 @@ template <bool GRAV, bool COL>
 __global__ void __launch_bounds__(HEAD_THREADS) k_walk_head(WalkArgs A) {
     __shared__ WalkHead H;
     __shared__ long long s_stat[HEAD_THREADS / 32][5];
-    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;
-    long long st[5] = {0, 0, 0, 0, 0};
     const int tid = threadIdx.x;
+    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) {
+        if (tid == 0) A.ctl->walk_head = -1;
+        return;
+    }
+    long long st[5] = {0, 0, 0, 0, 0};
     int nf = A.ctl->nd;
     if (tid < 5) H.n[tid] = 0;
     if (tid == 0) H.next[0] = H.bad[0] = 0;
@@ -669,28 +673,29 @@ __global__ void __launch_bounds__(WALK_THREADS) k_walk(WalkArgs A) {
     __shared__ int s_tmp[33];
     __shared__ WalkSlots S;
     __shared__ long long s_stat[WALK_WARPS][5];
-    if ((A.gate && *A.gate == 0) || aborted(A.ctl)) return;   // (every block, before the first barrier)
+    // Whether there is anything to walk is the head's word alone, which nothing writes during this launch, so
+    // that every block returns here or none does.  The error word would not do: the first generation, already
+    // more pairs than the head keeps, can fill a list and set it while a block has yet to start; that block
+    // would return, and the others wait for it at the barrier until their limit.
+    int it = A.ctl->walk_head;
+    if (it < 0) return;
     volatile int *vcount = A.fcount;
     unsigned bar = 0;
     long long st[5] = {0, 0, 0, 0, 0};   // decision statistics of this thread's pairs
-    int it = A.ctl->walk_head;
-    const bool head_bad = it < 0;
-    if (head_bad) it = 0;
-    else
-        for (; it < WALK_MAX_ITERS; it++) {
-            const int nf = min(vcount[it], A.front_cap);
-            if (nf == 0) break;
-            if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->walk_abort[(it + 1) % 3] = 0;   // slot of the next generation
-            walk_generation<GRAV, COL>(A, it, nf, st, S);
-            if (!grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
-            // overflow in this generation (slot it mod 3: identical for every block after the barrier)
-            if (((volatile int *)A.ctl->walk_abort)[it % 3]) { it++; break; }
-        }
+    for (; it < WALK_MAX_ITERS; it++) {
+        const int nf = min(vcount[it], A.front_cap);
+        if (nf == 0) break;
+        if (blockIdx.x == 0 && threadIdx.x == 0) A.ctl->walk_abort[(it + 1) % 3] = 0;   // slot of the next generation
+        walk_generation<GRAV, COL>(A, it, nf, st, S);
+        if (!grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
+        // overflow in this generation (slot it mod 3: identical for every block after the barrier)
+        if (((volatile int *)A.ctl->walk_abort)[it % 3]) { it++; break; }
+    }
     walk_stats<WALK_WARPS>(A, st, s_stat);
     // the collision statistics' copies below read every block's totals
     if (A.collisions && !grid_sync_on(&A.ctl->bar_walk, A.ctl, bar)) return;
     // the generation count and the barrier snapshot are the same in every block
-    if (A.gravity && !head_bad && it < WALK_MAX_ITERS && !((volatile int *)A.ctl->walk_abort)[(it + 2) % 3])
+    if (A.gravity && it < WALK_MAX_ITERS && !((volatile int *)A.ctl->walk_abort)[(it + 2) % 3])
         walk_lists(A, s_tmp, bar);
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         if (A.gravity) A.ctl->walk_iters = it;
