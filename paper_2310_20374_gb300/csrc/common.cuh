@@ -80,10 +80,11 @@ enum : int {
     ERR_DIRECTED = 64,    // directed list capacity exceeded
     ERR_LEVEL = 128,      // internal: tree deeper than MAX_LEVEL
     ERR_NONFINITE = 256,  // a position was NaN or infinite
+    ERR_NEAR = 512,       // near-field item capacity exceeded (n_near holds the number needed)
 };
 
 constexpr int ERR_ABORT_MASK =
-    ERR_CELLS | ERR_FRONTIER | ERR_M2L | ERR_P2P | ERR_TIMEOUT | ERR_DIRECTED | ERR_LEVEL | ERR_NONFINITE;
+    ERR_CELLS | ERR_FRONTIER | ERR_M2L | ERR_P2P | ERR_TIMEOUT | ERR_DIRECTED | ERR_LEVEL | ERR_NONFINITE | ERR_NEAR;
 
 // Device control block: counters written by kernels, read back by the host.
 struct Ctrl {

@@ -149,7 +149,7 @@ void alloc_cells(ncorp_ctx *c, int cap) {
     c->tree_valid = false;
 }
 
-void alloc_lists(ncorp_ctx *c, int front, int m2l, int p2p, int self) {
+void alloc_lists(ncorp_ctx *c, int front, int m2l, int p2p, int self, int near) {
     WalkLists &W = c->wl;
     if (front != W.front_cap) {
         W.front_cap = 0;
@@ -172,17 +172,17 @@ void alloc_lists(ncorp_ctx *c, int front, int m2l, int p2p, int self) {
         W.p2p_dir_cap = 0;
         dalloc(W.p2p, p2p);
         dalloc(W.self, self);
-        W.near_cap = 0;
         dalloc(W.p2p_src, 2 * static_cast<size_t>(p2p) + self);   // int2
-        // at most one item per NEAR_ENTRIES_MIN entries and two more per leaf, in lists that are far from
-        // full; a tree that needs more reports it like any full list
-        dalloc(W.near_items, static_cast<size_t>(p2p) / 4 + 2 * self);
-        W.near_cap = p2p / 4 + 2 * self;
         dalloc(W.cp2p, p2p);
         dalloc(W.cself, self);
         W.p2p_cap = p2p;
         W.self_cap = self;
         W.p2p_dir_cap = 2 * p2p + self;
+    }
+    if (near != W.near_cap) {
+        W.near_cap = 0;
+        dalloc(W.near_items, near);
+        W.near_cap = near;
     }
 }
 
@@ -236,9 +236,15 @@ void ensure_tree_capacity(ncorp_ctx *c, int n) {
         p2p = std::min(p2p, c->test_list_cap);
     }
     const int self = std::max(cc, c->floor_self);
-    if (c->wl.front_cap < front || c->wl.m2l_cap < m2l || c->wl.p2p_cap < p2p || c->wl.self_cap < self)
+    // Near-field items: an estimate.  A leaf's entries count once per subset of its moonlets (two subsets of 33 to
+    // 52 moonlets, one per 64 of more; FP64: one per 16 of up to 256) and are cut into shares of 4 (FP64: 12)
+    // entries or more, the smallest in the smallest trees.  Leaves of more than 64 moonlets at a small theta can
+    // need more, up to several items an entry: they then grow this list alone (n_near tells how many).
+    const int near = std::max(p2p / 2 + 2 * self, c->floor_near);
+    if (c->wl.front_cap < front || c->wl.m2l_cap < m2l || c->wl.p2p_cap < p2p || c->wl.self_cap < self ||
+        c->wl.near_cap < near)
         alloc_lists(c, std::max(front, c->wl.front_cap), std::max(m2l, c->wl.m2l_cap), std::max(p2p, c->wl.p2p_cap),
-                    std::max(self, c->wl.self_cap));
+                    std::max(self, c->wl.self_cap), std::max(near, c->wl.near_cap));
     int pc = std::max(1 << 16, 4 * n);
     if (c->test_pair_cap > 0) pc = std::min(pc, c->test_pair_cap);
     if (c->pair_cap < pc) alloc_pairs(c, pc);
@@ -284,7 +290,7 @@ bool grow_after(ncorp_ctx *c, int err) {
         grew = true;
     }
     WalkLists &W = c->wl;
-    int front = W.front_cap, m2l = W.m2l_cap, p2p = W.p2p_cap, self = W.self_cap;
+    int front = W.front_cap, m2l = W.m2l_cap, p2p = W.p2p_cap, self = W.self_cap, near = W.near_cap;
     if (err & ERR_FRONTIER) { front *= 2; grew = true; }
     if (err & (ERR_M2L | ERR_DIRECTED)) { m2l = std::max(2 * m2l, c->ctl_h->n_m2l + 1024); grew = true; }
     if (err & (ERR_P2P | ERR_DIRECTED)) {
@@ -292,13 +298,18 @@ bool grow_after(ncorp_ctx *c, int err) {
         self = std::max(2 * self, c->ctl_h->n_self + 1024);
         grew = true;
     }
+    if (err & ERR_NEAR) {   // (the walk counts every item it wants, also those without a place)
+        near = std::max({near + near / 8, c->ctl_h->n_near + c->ctl_h->n_near / 8 + 1024, c->floor_near});
+        grew = true;
+    }
     if (grew) {
-        alloc_lists(c, front, m2l, p2p, self);
+        alloc_lists(c, front, m2l, p2p, self, near);
         c->test_list_cap = 0;
         c->floor_front = std::max(c->floor_front, front);
         c->floor_m2l = std::max(c->floor_m2l, m2l);
         c->floor_p2p = std::max(c->floor_p2p, p2p);
         c->floor_self = std::max(c->floor_self, self);
+        c->floor_near = std::max(c->floor_near, near);
     }
     if (err & ERR_PAIRS) {
         c->test_pair_cap = 0;
@@ -2046,7 +2057,7 @@ int tune_forest(ncorp_batch *b, Forest &f) {
     f.tuned_n = f.n;
     b->tuned++;
     // the capacities the trials needed are not the chosen leaf size's
-    f.c->floor_cells = f.c->floor_front = f.c->floor_m2l = f.c->floor_p2p = f.c->floor_self = 0;
+    f.c->floor_cells = f.c->floor_front = f.c->floor_m2l = f.c->floor_p2p = f.c->floor_self = f.c->floor_near = 0;
     f.primed = false;
     return prime_forest(b, f);
 }

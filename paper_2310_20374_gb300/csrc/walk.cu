@@ -190,7 +190,7 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
                 const int f = __ldg(&A.first[i]), s0 = pp + xp;
                 int slot = s_items + xi;
                 if (slot + parts > A.near_cap || s0 + vp > A.p2p_dir_cap) {
-                    atomicOr(&A.ctl->err, ERR_DIRECTED);
+                    atomicOr(&A.ctl->err, slot + parts > A.near_cap ? ERR_NEAR : ERR_DIRECTED);
                 } else {
                     for (int t = 0; t < m; t += near_targets(m - t, A.fp64)) {
                         const int k = near_targets(m - t, A.fp64), np = near_shares(vp, k, n_leaves, A.fp64);
