@@ -228,9 +228,10 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {
 #pragma unroll
             for (int r = 0; r < 2; r++) {
                 const int j = W.moonlet(pos + 32 * r, lane);
-                // (a place past the window: a massless source far away; a last chunk is padded to quads)
-                ph[r] = j >= 0 ? A.hi4[j] : make_float4(1e9f, 0.f, 0.f, 0.f);
-                pl[r] = j >= 0 ? A.lo4[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+                // (a place past the window, which a last chunk's padding to quads sums: a massless source at one of
+                // the item's own moonlets, so that its separations are as finite as the leaf's)
+                ph[r] = j >= 0 ? A.hi4[j] : make_float4(th0.x, th0.y, th0.z, 0.f);
+                pl[r] = j >= 0 ? A.lo4[j] : tl0;
             }
         };
         if (at < I.s1) {
