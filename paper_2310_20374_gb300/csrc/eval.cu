@@ -45,6 +45,7 @@ struct EvalArgs {
     double *ax, *ay, *az;
     double *amx, *amy, *amz;
     double *nx, *ny, *nz;     // near-field sums per moonlet (tree order)
+    const uint64_t *key;      // sorted keys
     double kick_h;            // k_far: v += kick_h a after the evaluation (0: no kick)
     double *vx, *vy, *vz;
     const Ctrl *ctl;
@@ -309,6 +310,12 @@ __global__ void __launch_bounds__(32 * DESC_WARPS) k_descend(DescendArgs A) {
 // plus the near-field sums and the external forces: one thread per moonlet
 // in tree order (the moonlets of a leaf are consecutive, so the threads of a
 // warp read the same few expansions: broadcast loads).
+//
+// Coincident moonlets get one result, bit for bit: the first of them in tree
+// order computes it for all.  Their near-field sums, added up with atomics, differ in the last
+// bits, and moonlets at one place and velocity that part by one rounding would
+// throw each other apart.  They have equal keys, so only runs of equal keys
+// are searched, and one leaf (equal keys of two disks are no run).
 constexpr int FAR_THREADS = 256;
 
 template <int P, typename real>
@@ -321,6 +328,12 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far(EvalArgs A) {
         const int leaf = __ldg(&A.leaf_of[i]);
         const real *C = Cf + (size_t)leaf * NC;
         const double X = A.x[i], Y = A.y[i], Z = A.z[i];
+        const uint64_t key = __ldg(&A.key[i]);
+        auto in_run = [&](int j) { return j >= 0 && j < A.n && __ldg(&A.key[j]) == key && __ldg(&A.leaf_of[j]) == leaf; };
+        auto here = [&](int j) { return A.x[j] == X && A.y[j] == Y && A.z[j] == Z; };
+        int j = i - 1;
+        while (in_run(j) && !here(j)) j--;
+        if (in_run(j)) continue;   // moonlet j's thread writes this one's result
         double fx, fy, fz;   // the far field at the moonlet
         if constexpr (f32) {
             // the order-1 pair (hi in Cf, lo in Cf_lo) and the higher orders, added in FP64
@@ -347,14 +360,17 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far(EvalArgs A) {
         const double my = fy + A.ny[i];
         const double mz = fz + A.nz[i];
         const double gx = mx + ex, gy = my + ey, gz = mz + ez;
-        A.ax[i] = gx;
-        A.ay[i] = gy;
-        A.az[i] = gz;
-        if (A.amx) { A.amx[i] = mx; A.amy[i] = my; A.amz[i] = mz; }
-        if (A.kick_h != 0.0) {   // the step's closing half kick, as k_kick computes it
-            A.vx[i] = dadd(A.vx[i], dmul(A.kick_h, gx));
-            A.vy[i] = dadd(A.vy[i], dmul(A.kick_h, gy));
-            A.vz[i] = dadd(A.vz[i], dmul(A.kick_h, gz));
+        for (int k = i; k == i || in_run(k); k++) {
+            if (k != i && !here(k)) continue;
+            A.ax[k] = gx;
+            A.ay[k] = gy;
+            A.az[k] = gz;
+            if (A.amx) { A.amx[k] = mx; A.amy[k] = my; A.amz[k] = mz; }
+            if (A.kick_h != 0.0) {   // the step's closing half kick, as k_kick computes it
+                A.vx[k] = dadd(A.vx[k], dmul(A.kick_h, gx));
+                A.vy[k] = dadd(A.vy[k], dmul(A.kick_h, gy));
+                A.vz[k] = dadd(A.vz[k], dmul(A.kick_h, gz));
+            }
         }
     }
 }
@@ -418,6 +434,7 @@ static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, double G, ExtForce
     A.amy = want_mutual ? c->amy : nullptr;
     A.amz = want_mutual ? c->amz : nullptr;
     A.nx = c->amx; A.ny = c->amy; A.nz = c->amz;   // the far kernel overwrites them in place
+    A.key = P.key;
     A.ctl = c->ctl;
     A.kick_h = 0.0;
     A.vx = A.vy = A.vz = nullptr;
