@@ -530,8 +530,8 @@ __global__ void __launch_bounds__(RS_T) k_radix(RadixArgs A) {
 // order of equal keys is the order of places, and every (key, place) differs):
 // one cooperative launch with three grid barriers in place of the radix
 // sort's nine, bound by their latency and the loads between them.
-//   1. S = 8 B samples, spread evenly over the input in runs of four (a run is
-//      one sector), are ranked by counting, every block a share of them; every
+//   1. S = 8 B samples, spread over the input in runs of two (half the sectors
+//      of single ones), are ranked by counting, every block a share of them; every
 //      eighth of the ranked samples bounds a bucket;
 //   2. every key finds its bucket by binary search in shared memory and
 //      takes a place in its block's part of the bucket (an atomic in shared
@@ -553,6 +553,11 @@ __global__ void __launch_bounds__(RS_T) k_radix(RadixArgs A) {
 // ---------------------------------------------------------------------------
 constexpr int SS_T = RS_T, SS_BUCKETS = 1024, SS_OVER = 8, SS_CAP = 2048, SS_TARGETS = 4, SS_STAGE = 4096;
 constexpr int SS_MAX_N = SAMPLE_SORT_MAX;   // v0 holds bucket << 20 | place; 12 fraction bits of the sampling stride
+// Up to this many keys the samples are taken in runs of two, which is enough where a bucket may hold 8 averages; beyond
+// it a bucket may hold as few as 4, and two neighbours in the input count as little more than one sample where
+// the input is coherent (rows, rings): in a collision search of moonlets in rows of 128, N = 5.2e5 615 us with runs
+// of two and 533 with single samples, of a disk 797 and 811; at N = 1.2e5 314 and 305, of a disk 367 and 374.
+constexpr int SS_RUNS_MAX_N = 1 << 18;
 static_assert(SS_MAX_N <= 1 << 19 && SS_BUCKETS <= 1 << 11, "packing of bucket and place");
 
 struct SampleScratch {
@@ -573,9 +578,16 @@ __host__ __device__ inline int sample_buckets(int n) {
     return b < 1 ? 1 : (b > SS_BUCKETS ? SS_BUCKETS : b);
 }
 
-// Place of sample j of S in an input of n keys (n >= 4 S / 4 = S; S a multiple of four).
-__device__ __forceinline__ int sample_place(int j, unsigned stride) {
-    return 4 * static_cast<int>((static_cast<unsigned>(j >> 2) * stride) >> 12) + (j & 3);
+// Place of sample j of S in an input of n keys (n >= S): run j >> lg of 2^lg samples lies anywhere in its share of the
+// input, by a hash of its number.  At a fixed stride the runs fell on the same columns of moonlets stored in rows or
+// ring by ring and split them so badly that the call went on to the radix sort: the static sort of 16384 moonlets in
+// rows of 64 took 122 us (radix alone 101, now 48), of 65536 135 (125, now 72).
+__device__ __forceinline__ int sample_place(int j, unsigned stride, int lg) {
+    const unsigned r = static_cast<unsigned>(j) >> lg;
+    const unsigned a = (r * stride) >> 12, room = ((r + 1) * stride >> 12) - a;   // room >= 1
+    unsigned h = (r + 1) * 0x9e3779b1u;
+    h = (h ^ h >> 15) * 0x85ebca77u;
+    return static_cast<int>((a + __umulhi(h ^ h >> 13, room)) << lg) + (j & ((1 << lg) - 1));
 }
 
 struct SampleSplit {
@@ -607,7 +619,8 @@ __global__ void __launch_bounds__(SS_T) k_sample(SampleArgs A) {
     if (b == 0)
         for (int i = tid; i < B; i += SS_T) A.scr->count[i] = 0;
     if (B > 1) {
-        const unsigned stride = (static_cast<unsigned>(n / 4) << 12) / static_cast<unsigned>(S / 4);
+        const int lg = n > SS_RUNS_MAX_N ? 0 : 1;
+        const unsigned stride = (static_cast<unsigned>(n >> lg) << 12) / static_cast<unsigned>(S >> lg);
         constexpr int PER_BLOCK = SS_T / 32 * SS_TARGETS;
         for (int r0 = 0; r0 < S; r0 += G * PER_BLOCK) {
             if (r0 + b * SS_TARGETS >= S) break;   // (the same for the whole block)
@@ -617,13 +630,13 @@ __global__ void __launch_bounds__(SS_T) k_sample(SampleArgs A) {
             int acc[SS_TARGETS];
 #pragma unroll
             for (int u = 0; u < SS_TARGETS; u++) {
-                t[u] = act ? R.k0[sample_place(i0 + u, stride)] : 0ull;
+                t[u] = act ? R.k0[sample_place(i0 + u, stride, lg)] : 0ull;
                 acc[u] = 0;
             }
             for (int c0 = 0; c0 < S; c0 += SS_STAGE) {
                 const int m = min(SS_STAGE, S - c0);
                 __syncthreads();
-                for (int j = tid; j < m; j += SS_T) U.sample[j] = R.k0[sample_place(c0 + j, stride)];
+                for (int j = tid; j < m; j += SS_T) U.sample[j] = R.k0[sample_place(c0 + j, stride, lg)];
                 __syncthreads();
                 if (!act) continue;
                 // samples before the targets count if not larger, those after them if smaller
@@ -648,7 +661,7 @@ __global__ void __launch_bounds__(SS_T) k_sample(SampleArgs A) {
                 const int rank = static_cast<int>(__reduce_add_sync(0xffffffffu, static_cast<unsigned>(acc[u])));
                 if (act && lane == 0 && rank > 0 && rank % SS_OVER == 0) {
                     A.scr->skey[rank / SS_OVER] = t[u];
-                    A.scr->spos[rank / SS_OVER] = static_cast<unsigned>(sample_place(i0 + u, stride));
+                    A.scr->spos[rank / SS_OVER] = static_cast<unsigned>(sample_place(i0 + u, stride, lg));
                 }
             }
         }
