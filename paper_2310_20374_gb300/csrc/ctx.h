@@ -303,7 +303,7 @@ namespace ncorp {
 void launch_bbox_keys(ncorp_ctx *c, const double *x, const double *y, const double *z, int n, uint64_t *key,
                       uint32_t *qx, uint32_t *qy, uint32_t *qz, bool bbox_done = false, const int *gate = nullptr);
 // by_disk: the keys are a forest's moonlet keys (every disk's own root cube); they are sorted by (disk, key)
-constexpr int SAMPLE_SORT_MAX = 1 << 19;   // most keys the sample sort takes
+constexpr int SAMPLE_SORT_MAX = 7 << 16;   // most keys the sample sort takes (why: sort.cu)
 void sort_u64(ncorp_ctx *c, uint64_t *keys, uint32_t *vals, uint64_t *keys_alt, uint32_t *vals_alt, int n,
                     int bits, bool bar_zeroed = false, const int *gate = nullptr, bool by_disk = false);
 // spec_dt > 0 (fused walk): also the bounds on next step's R + dt |v| of the current tree set's moonlets,

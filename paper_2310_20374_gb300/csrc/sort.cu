@@ -546,10 +546,14 @@ __global__ void __launch_bounds__(RS_T) k_radix(RadixArgs A) {
 // the search and the sample ranking with their number, at most 1024).
 // With eight samples a bucket the largest of a thousand buckets is about 2.7
 // averages; a bucket above SS_CAP (keys that differ only between the samples)
-// sends the call to the radix sort, in the same launch.  Measured: N = 4e3 9 us,
-// 6.5e4 17, 1.2e5 26, 2e5 44 (ranks 10, search 9, moves 4, buckets 13, barriers), 5.2e5 102; the radix sort's
-// eight passes take 51, 84, 101, 117 and 149.  Past SS_MAX_N the buckets' counting, which grows with their size,
-// would overtake the radix passes.
+// sends the call to the radix sort, in the same launch.  The kernel alone on a
+// disk's keys, caches cold: N = 4e3 14 us, 6.6e4 35, 1.2e5 44, 2e5 59, 4e5 84,
+// 4.6e5 126; the radix sort's eight passes take 55, 81, 91, 99, 112 and 144.
+// Past SS_MAX_N the buckets' counting, which grows with the square of their
+// size, overtakes the radix passes: the sort stage of a collision search (box,
+// keys, sort, gather; three disks and a ball) takes 201..213 us with the sample
+// sort and 218..220 with the radix sort at 4.6e5, 216..250 and 224..226 at
+// 4.9e5, 234..250 and 230 at 5.2e5.
 // ---------------------------------------------------------------------------
 constexpr int SS_T = RS_T, SS_BUCKETS = 1024, SS_OVER = 8, SS_CAP = 2048, SS_TARGETS = 4, SS_STAGE = 4096;
 constexpr int SS_MAX_N = SAMPLE_SORT_MAX;   // v0 holds bucket << 20 | place; 12 fraction bits of the sampling stride

@@ -72,6 +72,24 @@ def sample_places(n):
     return (first[:, None] + np.arange(1 << lg, dtype=np.uint64)).ravel().astype(np.int64)
 
 
+@pytest.mark.parametrize("n", [1 << 18, (1 << 18) + 1, 7 << 16, (7 << 16) + 1])
+def test_order_beside_the_lines(n):
+    """On both sides of the most keys sampled in runs, and of the most the sample sort takes."""
+    import torch
+    from paper_2310_20374_gb300 import ncorp
+    pos = np.random.default_rng(n).uniform(-1.0, 1.0, (n, 3))
+    pos[:n // 8] = pos[n // 8:2 * (n // 8)]   # some places twice
+    ctx = ncorp.ncorp_init(ncorp.ncorp_config_default(), n, 0, torch.cuda.current_stream().cuda_stream)
+    try:
+        order = np.zeros(n, dtype=np.int64)
+        ncorp.ncorp_accel(ctx, pos, np.full(n, 1.0 / n), n, 1, 0.5, np.zeros((n, 3)))
+        ncorp.ncorp_tree_export(ctx, order=order)
+    finally:
+        ncorp.ncorp_free(ctx)
+    want = np.asarray(oracle.keys(pos)[2]).astype(np.uint64)
+    assert np.array_equal(order, np.argsort(want, kind="stable"))
+
+
 @pytest.mark.parametrize("n", [4000, 20011, 65536, 131072, 300001])
 def test_keys_between_the_samples(n):
     """All keys but the samples in one octant's corner: more than a bucket holds."""
