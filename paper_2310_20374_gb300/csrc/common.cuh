@@ -93,7 +93,6 @@ struct Ctrl {
     int n_leaves;
     int max_level;
     int level_start[MAX_LEVEL + 3];
-    int frontier_count[2];
     int n_m2l;             // unordered well-separated pairs
     int n_p2p;             // leaf-leaf direct pairs
     int n_self;            // leaves interacting with themselves
@@ -267,24 +266,6 @@ __device__ __forceinline__ bool grid_sync(Ctrl *ctl, unsigned &passed) { return 
 
 // ---- warp helpers -----------------------------------------------------------
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
-
-// Warp-aggregated append: every active lane wants `k` slots in a list whose
-// length is *counter; returns the lane's first slot (slots >= cap must be
-// treated as overflow by the caller).  All lanes of the warp must call it.
-__device__ __forceinline__ int warp_append(int *counter, int k) {
-    unsigned lane = lane_id();
-    int incl = k;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        int v = __shfl_up_sync(0xffffffffu, incl, o);
-        if ((int)lane >= o) incl += v;
-    }
-    int total = __shfl_sync(0xffffffffu, incl, 31);
-    int base = 0;
-    if (lane == 31 && total > 0) base = atomicAdd(counter, total);
-    base = __shfl_sync(0xffffffffu, base, 31);
-    return base + incl - k;
-}
 
 __device__ __forceinline__ int warp_sum(int v) {
 #pragma unroll

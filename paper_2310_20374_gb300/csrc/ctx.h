@@ -28,7 +28,7 @@ constexpr int BLOCKSUM_INTS = 8192;
 struct Cells {
     int cap = 0;
     int *level = nullptr, *first = nullptr, *count = nullptr, *child0 = nullptr, *nchild = nullptr,
-        *parent = nullptr, *arrive = nullptr, *arrive_m = nullptr;   // arrival counters: collision climb, multipoles
+        *parent = nullptr, *arrive_m = nullptr;   // arrive_m: arrival counters of the multipoles
     uint32_t *cx = nullptr, *cy = nullptr, *cz = nullptr;
     double *M = nullptr, *sx = nullptr, *sy = nullptr, *sz = nullptr, *rmax = nullptr, *rcrit = nullptr,
            *rho = nullptr;                                 // gravity climb
@@ -344,7 +344,7 @@ struct ExtForce {
 // multipoles are computed: S.ax = mutual + external, amx = mutual (want_mutual)
 void launch_standard(ncorp_ctx *c, const ParticleSet &S, int n, int p, bool mixed, double G, ExtForce ext,
                      bool want_mutual, int pre, int post);
-void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G, ExtForce ext, bool want_mutual,
+void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, ExtForce ext, bool want_mutual,
                 double kick_h = 0.0);
 
 // ---- near.cu ----

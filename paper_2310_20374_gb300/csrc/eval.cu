@@ -33,14 +33,13 @@ __constant__ ExpTable2 c_exp2 = make_exp_table2();
 
 struct EvalArgs {
     int n;                     // moonlets of the tree
-    const int *leaves, *level, *parent, *first, *count, *leaf_of;
+    const int *leaf_of;
     const double *sx, *sy, *sz, *rho;
     const float4 *gh, *gl;
     const void *Cf;   // complete local expansions
     const float *Cf_lo;   // mixed: low parts of their order-1 coefficients
-    const double *x, *y, *z, *m;
+    const double *x, *y, *z;
     const float4 *hi4, *lo4;
-    double G;
     ExtForce ext;
     double *ax, *ay, *az;
     double *amx, *amy, *amz;
@@ -415,19 +414,17 @@ void launch_descend(ncorp_ctx *c, int p, bool mixed) {
 #undef NCORP_DESC_CASE
 }
 
-static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, double G, ExtForce ext, bool want_mutual) {
+static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, ExtForce ext, bool want_mutual) {
     Cells &C = c->cells;
     EvalArgs A;
     A.n = c->cur_n;
-    A.leaves = C.leaves; A.level = C.level; A.parent = C.parent; A.first = C.first; A.count = C.count;
     A.leaf_of = C.leaf_of;
     A.sx = C.sx; A.sy = C.sy; A.sz = C.sz; A.rho = C.rho;
     A.gh = C.gh; A.gl = C.gl;
     A.Cf = C.Cf;
     A.Cf_lo = C.Cf_lo;
-    A.x = P.x; A.y = P.y; A.z = P.z; A.m = P.m;
+    A.x = P.x; A.y = P.y; A.z = P.z;
     A.hi4 = P.hi4; A.lo4 = P.lo4;
-    A.G = G;
     A.ext = ext;
     A.ax = P.ax; A.ay = P.ay; A.az = P.az;
     A.amx = want_mutual ? c->amx : nullptr;
@@ -441,9 +438,9 @@ static EvalArgs eval_args(ncorp_ctx *c, const ParticleSet &P, double G, ExtForce
     return A;
 }
 
-void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, double G, ExtForce ext, bool want_mutual,
+void launch_far(ncorp_ctx *c, const ParticleSet &P, int p, bool mixed, ExtForce ext, bool want_mutual,
                 double kick_h) {
-    EvalArgs A = eval_args(c, P, G, ext, want_mutual);
+    EvalArgs A = eval_args(c, P, ext, want_mutual);
     A.kick_h = kick_h;
     A.vx = P.vx; A.vy = P.vy; A.vz = P.vz;
 #define NCORP_FAR_CASE(PP)                       \

@@ -116,7 +116,7 @@ void alloc_cells(ncorp_ctx *c, int cap) {
     C.cap = 0;
     c->tree_valid = false;
     dalloc(C.level, cap); dalloc(C.first, cap); dalloc(C.count, cap); dalloc(C.child0, cap);
-    dalloc(C.nchild, cap); dalloc(C.parent, cap); dalloc(C.arrive, cap); dalloc(C.arrive_m, cap);
+    dalloc(C.nchild, cap); dalloc(C.parent, cap); dalloc(C.arrive_m, cap);
     dalloc(C.cx, cap); dalloc(C.cy, cap); dalloc(C.cz, cap);
     dalloc(C.M, cap); dalloc(C.sx, cap); dalloc(C.sy, cap); dalloc(C.sz, cap);
     dalloc(C.rmax, cap); dalloc(C.rcrit, cap); dalloc(C.rho, cap);
@@ -681,7 +681,7 @@ void gravity(ncorp_ctx *c, ParticleSet &S, int p, double theta, double t, bool w
     { Stage st(c, NCORP_STAGE_M2L); launch_m2l(c, p, mixed); }
     { Stage st(c, NCORP_STAGE_DESCEND); launch_descend(c, p, mixed); }
     NCORP_CUDA_CHECK(cudaStreamWaitEvent(c->stream, c->ev_near, 0));
-    { Stage st(c, NCORP_STAGE_EVAL); launch_far(c, S, p, mixed, G, external(c, t), want_mutual, kick_h); }
+    { Stage st(c, NCORP_STAGE_EVAL); launch_far(c, S, p, mixed, external(c, t), want_mutual, kick_h); }
 }
 
 // Gravity of the tree in the current set by the standard tree code: the
@@ -1580,7 +1580,7 @@ void ncorp_free(ncorp_ctx *c) {
     for (int set = 0; set < 2; set++) {
         Cells &C = c->cells;
         dfree(C.level); dfree(C.first); dfree(C.count); dfree(C.child0); dfree(C.nchild); dfree(C.parent);
-        dfree(C.arrive); dfree(C.arrive_m); dfree(C.cx); dfree(C.cy); dfree(C.cz); dfree(C.M); dfree(C.sx); dfree(C.sy); dfree(C.sz);
+        dfree(C.arrive_m); dfree(C.cx); dfree(C.cy); dfree(C.cz); dfree(C.M); dfree(C.sx); dfree(C.sy); dfree(C.sz);
         dfree(C.rmax); dfree(C.rcrit); dfree(C.rho); dfree(C.bx); dfree(C.by); dfree(C.bz); dfree(C.bmax);
         dfree(C.bcrit); dfree(C.gh); dfree(C.gl); dfree(C.bh); dfree(C.bl); dfree(C.Mh); dfree(C.Ch); dfree(C.Cf); dfree(C.Cf_lo); dfree(C.Ch_lo);
         dfree(C.leaves); dfree(C.leaf_of); dfree(C.rc_spec); dfree(C.blocksum); dfree(C.done);

@@ -166,17 +166,6 @@ __device__ __forceinline__ void p2p_f32x2(f32x2 hx, f32x2 hy, f32x2 hz, f32x2 mu
     az = fma2(dz, f3, az);
 }
 
-// df_add (fields.cuh) on both halves
-__device__ __forceinline__ void df_add2(f32x2 &hi, f32x2 &lo, f32x2 b) {
-    const f32x2 neg = pack2(-1.0f, -1.0f);   // x - y as fma(y, -1, x): one rounding
-    const f32x2 s = add2(hi, b);
-    const f32x2 bv = fma2(hi, neg, s);
-    const f32x2 e = add2(fma2(fma2(bv, neg, s), neg, hi), fma2(bv, neg, b));
-    const f32x2 l = add2(lo, e);
-    hi = add2(s, l);
-    lo = fma2(fma2(s, neg, hi), neg, l);
-}
-
 constexpr int NEAR_CHUNK = 64;   // sources a warp stages at a time
 
 __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {

@@ -62,7 +62,7 @@ struct BuildArgs {
     const uint64_t *key;
     const uint32_t *qx, *qy, *qz;
     int n, s, cap, chunk;   // chunk: moonlets per block, a multiple of BUILD_T
-    int *level, *first, *count, *child0, *nchild, *parent, *arrive, *arrive_m;
+    int *level, *first, *count, *child0, *nchild, *parent, *arrive_m;
     uint32_t *cx, *cy, *cz;
     int *wcnt, *woff;       // the walk's per-cell counts [cap + 1], zeroed for it
     int *leaves, *leaf_of;  // leaf_of[i] first holds moonlet i's levels, (L0 << 8 | Lmax) or -1
@@ -258,8 +258,7 @@ __global__ void __launch_bounds__(BUILD_T) k_build(BuildArgs A) {
                     A.first[c] = i;
                     A.child0[c] = L < Lmax ? upto(L + 1) : -1;
                     A.parent[c] = par;
-                    A.arrive[c] = 0;     // arrival counters of the multipoles, zeroed as cells are made
-                    A.arrive_m[c] = 0;
+                    A.arrive_m[c] = 0;   // arrival counters of the multipoles, zeroed as cells are made
                     A.cx[c] = qx >> (KEY_BITS - L);
                     A.cy[c] = qy >> (KEY_BITS - L);
                     A.cz[c] = qz >> (KEY_BITS - L);
@@ -298,7 +297,7 @@ void launch_build(ncorp_ctx *c, const ParticleSet &P, int n, int s, const int *g
     A.n = n; A.s = s; A.cap = C.cap;
     A.level = C.level; A.first = C.first; A.count = C.count; A.child0 = C.child0; A.nchild = C.nchild;
     A.parent = C.parent; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
-    A.arrive = C.arrive; A.arrive_m = C.arrive_m;
+    A.arrive_m = C.arrive_m;
     A.leaves = C.leaves; A.leaf_of = C.leaf_of;
     A.wcnt = c->wl.cnt; A.woff = c->wl.p2p_off;
     A.bcount = C.blocksum; A.ctl = c->ctl;
@@ -400,7 +399,7 @@ struct ClimbArgs {
     const double *x, *y, *z, *m;
     const float4 *hi4, *lo4;
     const double *vx, *vy, *vz, *R;
-    int *first, *count, *child0, *nchild, *parent, *level, *arrive;
+    int *first, *count, *child0, *nchild, *parent, *level;
     uint32_t *cx, *cy, *cz;
     double *M, *sx, *sy, *sz, *rmax, *rcrit, *rho;
     float4 *gh, *gl;
@@ -417,13 +416,6 @@ struct ClimbArgs {
 };
 
 constexpr int CLIMB_WARPS_COOP = 8;
-
-template <typename real>
-__device__ __forceinline__ real warp_sum_r(real v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
 
 // ---- leaves: eight leaves per warp, four lanes per leaf.  The centre's
 // sums run in the oracle's order, one sum per lane (q = 0: the weights,
@@ -583,16 +575,6 @@ __device__ __forceinline__ void p2m_add(real dx, real dy, real dz, real mu, real
         for (int k = 0; k <= n; k++)
 #pragma unroll
             for (int c = 0; c <= k; c++) acc[midx(n - k, k - c, c)] += mu * px[n - k] * py[k - c] * pz[c];
-}
-
-template <int P, typename real>
-__device__ __forceinline__ void store_reduced(real *acc, real *dst, int lane) {
-    constexpr int NM = num_m(P);
-#pragma unroll
-    for (int j = 0; j < NM; j++) {
-        const real v = warp_sum_r(acc[j]);
-        if (lane == (j & 31)) dst[j] = v;
-    }
 }
 
 // ---- gravity geometry of parents from their children (Eqs. expansion_center,
@@ -1019,7 +1001,7 @@ void launch_climb_geometry(ncorp_ctx *c, const ParticleSet &P, double G, double 
     ClimbArgs A{};
     A.x = P.x; A.y = P.y; A.z = P.z; A.m = P.m; A.hi4 = P.hi4; A.lo4 = P.lo4;
     A.first = C.first; A.count = C.count; A.child0 = C.child0; A.nchild = C.nchild; A.parent = C.parent;
-    A.level = C.level; A.arrive = C.arrive; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
+    A.level = C.level; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
     A.M = C.M; A.sx = C.sx; A.sy = C.sy; A.sz = C.sz; A.rmax = C.rmax; A.rcrit = C.rcrit; A.rho = C.rho;
     A.gh = C.gh; A.gl = C.gl;
     A.Mh = C.Mh; A.leaves = C.leaves; A.ctl = c->ctl; A.G = G; A.theta = theta; A.cap = C.cap;
@@ -1254,7 +1236,7 @@ void launch_climb_collision(ncorp_ctx *c, const ParticleSet &P, const double *vx
     A.x = P.x; A.y = P.y; A.z = P.z; A.R = P.R; A.vx = vx; A.vy = vy; A.vz = vz;
     A.hi4 = P.hi4; A.lo4 = P.lo4;
     A.first = C.first; A.count = C.count; A.child0 = C.child0; A.nchild = C.nchild; A.parent = C.parent;
-    A.level = C.level; A.arrive = C.arrive; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
+    A.level = C.level; A.cx = C.cx; A.cy = C.cy; A.cz = C.cz;
     A.sx = C.bx; A.sy = C.by; A.sz = C.bz; A.rmax = C.bmax; A.rcrit = C.bcrit;
     A.gh = C.bh; A.gl = C.bl;
     A.leaves = C.leaves; A.ctl = c->ctl; A.dt = dt; A.cv4 = c->cv4;
