@@ -46,7 +46,7 @@ struct CollideArgs {
     const int *first, *count;
     const double *x, *y, *z, *vx, *vy, *vz, *R;
     const float4 *hi4, *lo4;
-    const float4 *cv;          // velocity rounded to FP32 (xyz), R + dt |v| rounded up to FP32 (w)
+    const float4 *cv;          // velocity cut (or rounded) to FP32 (xyz), an upper bound of R + dt |v| (w)
     const float4 *bh, *bl;     // per cell: collision centre hi (xyz) and r_crit in FP32 (w); centre lo
     const int *perm;
     double dt;
@@ -83,12 +83,15 @@ __device__ __forceinline__ void test_and_emit(const CollideArgs &A, int u, int v
 //     dt_c in [0, dt], so the least distance over [0, dt] is at most R1 + R2:
 //     with t* = clamp(-dr.dv / dv^2, 0, dt), |dr + t* dv|^2 against
 //     (R1 + R2)^2 (1 + 2^-9) plus 2^-12 (|dr|^2 + dt^2 |dv|^2) plus 1025
-//     delta^2.  delta = dt 2^-23 (|v1| + |v2|, sums of components) is what the velocities'
-//     rounding to FP32 can move a trajectory by, so also the least distance (where |dv| is
-//     below the velocities' FP32 resolution it is all that dv says):
-//     (Rs + delta)^2 <= Rs^2 (1 + 2^-10) + 1025 delta^2.  The margin
-//     exceeds the FP32 evaluation's error (the terms of the quadratic are bounded by that
-//     scale) by orders of magnitude, and the FP64 predicate's rounding likewise.
+//     delta^2.  delta = dt 2^-23 (|v1| + |v2|, sums of components) is what the
+//     velocities' FP32 copies can move a trajectory by, so also the least
+//     distance (where |dv| is below their resolution it is all that dv says).
+//     The collision climb cuts them: an error below 2^-23 of a component, which
+//     delta takes without a margin of its own (a fused step rounds them: half).
+//     (Rs + delta)^2 <= Rs^2 (1 + 2^-10) + 1025 delta^2.  The other margins
+//     exceed the FP32 evaluation's error (the terms of the quadratic are bounded
+//     by that scale) by orders of magnitude, and the FP64 predicate's rounding
+//     likewise.
 __device__ __forceinline__ bool may_touch(const float4 &h, const float4 &l, float r, const float4 &th,
                                           const float4 &tl, float tr, float &dx, float &dy, float &dz) {
     dx = (h.x - th.x) + (l.x - tl.x);
@@ -111,12 +114,16 @@ __device__ __forceinline__ bool may_meet(float dx, float dy, float dz, const flo
     return ex * ex + ey * ey + ez * ez <= Rs * Rs * (1.0f + 0x1p-9f) + margin;
 }
 
-// A pair that overlaps already cannot collide: with dr^2 < (R1 + R2)^2 Delta exceeds (dr.dv)^2, so dt_c < 0.  In FP32
-// with a margin of 2^-7 on the squares (both are good to 2^-18), where Delta exceeds (dr.dv)^2 by 2^-7 of itself and
-// the FP64 test's rounding cannot turn the sign; not where the separation or dv is near the resolution of the
-// positions' FP32 pairs (s: a bound on the position's size) or the squares near FP32's range.  In a dense ring most pairs
-// that pass test 2 overlap, and each sent its warp through some 3000 cycles of the FP64 pipe (60 % busy): with this and
-// radius_f32 the kernel alone goes from 275 to 148 us on a ring of N = 2e5, from 100 to 48 in the step with impacts at 3e4.
+// A pair that overlaps already cannot collide: with dr^2 < (R1 + R2)^2 Delta
+// exceeds (dr.dv)^2, so dt_c < 0.  In FP32 with a margin of 2^-7 on the squares
+// (both are good to 2^-18), where Delta exceeds (dr.dv)^2 by 2^-7 of itself and
+// the FP64 test's rounding cannot turn the sign; not where the separation or dv
+// is near the resolution of the positions' FP32 pairs (s: a bound on the
+// position's size) or the squares near FP32's range.  In a dense ring most
+// pairs that pass test 2 overlap, and each sent its warp through some 3000
+// cycles of the FP64 pipe (60 % busy): with this and radius_f32 the kernel
+// alone goes from 275 to 148 us on a ring of N = 2e5, from 100 to 48 in the
+// step with impacts at 3e4.
 __device__ __forceinline__ bool overlapping(float dx, float dy, float dz, const float4 &v, const float4 &tv, float Rs,
                                             float s) {
     const float ux = v.x - tv.x, uy = v.y - tv.y, uz = v.z - tv.z;
@@ -124,8 +131,9 @@ __device__ __forceinline__ bool overlapping(float dx, float dy, float dz, const 
     return d2 < R2 * (1.0f - 0x1p-7f) && R2 > 1e-24f && R2 < 1e30f && Rs > 0x1p-30f * s && u2 > 1e-20f;
 }
 
-// A radius in FP32, at most 2^-23 of it below: cut by integer instructions (a conversion takes the FP64 pipe; three of
-// them per item were a fifth of its time).
+// A radius in FP32, at most 2^-23 of it below: cut by integer instructions (a
+// conversion takes the FP64 pipe; three of them per item were a fifth of its
+// time).
 __device__ __forceinline__ float radius_f32(double R) {
     const unsigned hi = static_cast<unsigned>(__double2hiint(R)), lo = static_cast<unsigned>(__double2loint(R));
     if ((hi >> 20) - 897u < 254u) return __uint_as_float(((hi - (896u << 20)) << 3) | (lo >> 29));
@@ -241,9 +249,11 @@ __global__ void __launch_bounds__(32 * COL_WARPS, 4) k_collide(CollideArgs A) {
                     for (int k = g; k < cnt; k += G) {
                         const int v = s_j[wl][k];
                         float dx, dy, dz;
-                        if ((!self || v > u) && may_touch(s_h[wl][k], s_l[wl][k], s_v[wl][k].w, th, tl, tv.w, dx, dy, dz) &&
+                        if ((!self || v > u) &&
+                            may_touch(s_h[wl][k], s_l[wl][k], s_v[wl][k].w, th, tl, tv.w, dx, dy, dz) &&
                             may_meet(dx, dy, dz, s_v[wl][k], tv, (s_R[wl][k] + tR) * (1.0f + 0x1p-20f), dtf) &&
-                            !overlapping(dx, dy, dz, s_v[wl][k], tv, s_R[wl][k] + tR, fabsf(th.x) + fabsf(th.y) + fabsf(th.z)))
+                            !overlapping(dx, dy, dz, s_v[wl][k], tv, s_R[wl][k] + tR,
+                                         fabsf(th.x) + fabsf(th.y) + fabsf(th.z)))
                             test_and_emit(A, ft + u, fs + v);
                     }
                 }

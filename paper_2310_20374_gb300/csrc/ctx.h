@@ -87,9 +87,10 @@ constexpr int WALK_MAX_ITERS = 96;
 // direct entries.  The mixed kernel takes an item's m targets two per lane in
 // G = floor(32 / ceil(m / 2)) groups, so 33 to 52 targets (one group, 52 to 81 %
 // of the lanes) go better as 32 (two groups, every lane) and the rest, although
-// the sources are then staged twice.
-// The FP64 kernel takes all of a leaf's entries and few targets: its lanes hold the sources, which few entries
-// would not fill, and a warp instruction takes so long that an item must be few of them.
+// the sources are then staged twice.  The FP64 kernel takes many of a leaf's
+// entries and few targets: its lanes hold the sources, which few entries would
+// not fill, and a warp instruction takes so long that an item must be few of
+// them.
 constexpr int NEAR64_TARGETS = 16;   // (64 in leaves of more than 256, to bound the items)
 __host__ __device__ inline int near_targets(int m, bool fp64) {
     if (m > (fp64 ? 256 : 64)) return 64;
@@ -107,7 +108,7 @@ __host__ __device__ inline int near_targets(int m, bool fp64) {
 // about that of four).
 constexpr int NEAR_ENTRIES = 10, NEAR_ENTRIES_MIN = 4, NEAR_ITEMS_WANTED = 8192;
 __host__ __device__ inline int near_shares(int E, int m, int n_leaves, bool fp64) {
-    if (fp64) {   // 12 to 96 entries, by the leaves: 425 to 407 us a step at N = 1e4 (48: 504), 5160 to 4130 at 1e5 (32: 4250)
+    if (fp64) {   // 12 to 96 entries, by the leaves (a step at N = 1e4: 407 us, 48 entries 504; at 1e5 4130, 32 4250)
         const int per = n_leaves / 48 < 12 ? 12 : (n_leaves / 48 > 96 ? 96 : n_leaves / 48);
         return (E + per - 1) / per;
     }
@@ -222,8 +223,8 @@ struct ncorp_ctx {
 
     ncorp::ParticleSet A, B, Cset;   // A: resident state; B: scratch (half-kicked v, drifted x); Cset: next order
     double *amx = nullptr, *amy = nullptr, *amz = nullptr;   // mutual acceleration (tree order)
-    float4 *cv4 = nullptr;           // collision search, per moonlet: velocity rounded to FP32 (xyz) and
-                                     // R + dt |v| rounded up (w)
+    float4 *cv4 = nullptr;           // collision search, per moonlet: velocity in FP32, cut by the collision climb
+                                     // (rounded by a fused step's kick-drift) (xyz), an upper bound of R + dt |v| (w)
     uint64_t *key_alt = nullptr;
     uint64_t *resort_mkey = nullptr;   // nearly-sorted key sort: movers and per-block counts
     uint32_t *resort_midx = nullptr;

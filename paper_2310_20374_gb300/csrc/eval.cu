@@ -311,10 +311,11 @@ __global__ void __launch_bounds__(32 * DESC_WARPS) k_descend(DescendArgs A) {
 // warp read the same few expansions: broadcast loads).
 //
 // Coincident moonlets get one result, bit for bit: the first of them in tree
-// order computes it for all.  Their near-field sums, added up with atomics, differ in the last
-// bits, and moonlets at one place and velocity that part by one rounding would
-// throw each other apart.  They have equal keys, so only runs of equal keys
-// are searched, and one leaf (equal keys of two disks are no run).
+// order computes it for all.  Their near-field sums, added up with atomics,
+// differ in the last bits, and moonlets at one place and velocity that part by
+// one rounding would throw each other apart.  They have equal keys, so only
+// runs of equal keys are searched, and one leaf (equal keys of two disks are no
+// run).
 constexpr int FAR_THREADS = 256;
 
 template <int P, typename real>
@@ -328,7 +329,9 @@ __global__ void __launch_bounds__(FAR_THREADS) k_far(EvalArgs A) {
         const real *C = Cf + (size_t)leaf * NC;
         const double X = A.x[i], Y = A.y[i], Z = A.z[i];
         const uint64_t key = __ldg(&A.key[i]);
-        auto in_run = [&](int j) { return j >= 0 && j < A.n && __ldg(&A.key[j]) == key && __ldg(&A.leaf_of[j]) == leaf; };
+        auto in_run = [&](int j) {
+            return j >= 0 && j < A.n && __ldg(&A.key[j]) == key && __ldg(&A.leaf_of[j]) == leaf;
+        };
         auto here = [&](int j) { return A.x[j] == X && A.y[j] == Y && A.z[j] == Z; };
         int j = i - 1;
         while (in_run(j) && !here(j)) j--;

@@ -24,12 +24,13 @@
 //
 // Work layout: the directed entries (target, source) are grouped by target.
 // One warp per target cell: the lanes take the target's sources in turn, each
-// accumulating the target's coefficients in registers; a butterfly reduction
-// then leaves the sums on every lane, and each lane stores its share of the
-// coefficients (the warp owns the target, so no atomics are needed; targets
-// without entries get zeros).  Both directions of a pair are evaluated
-// (A <- B and B <- A), which is the symmetric treatment of Sect. 3.4.3 split
-// into its two halves.
+// accumulating the target's coefficients in registers.  The lanes' sums are
+// added 32 coefficients at a time, by halving (lane_sums): lane l is left with
+// coefficient g + l of group g and stores that one; only the double-float
+// order-1 terms of the mixed form take a butterfly (the warp owns the target,
+// so no atomics are needed; targets without entries get zeros).  Both
+// directions of a pair are evaluated (A <- B and B <- A), which is the
+// symmetric treatment of Sect. 3.4.3 split into its two halves.
 #include "ctx.h"
 #include "fields.cuh"
 

@@ -107,8 +107,9 @@ __device__ __forceinline__ void near_store(const NearArgs &A, int i, bool whole,
 // operations per issue slot, the same rounding as the scalar ones): 15 issue
 // slots a pair, below the pipe's 21 cycles.  The next chunk's positions are
 // loaded into registers before the current chunk is summed.  Measured alone:
-// 207 -> 161 us at N = 1e5, p = 6 (61 % of the issue slots and 60 % of the FP32
-// pipe busy, 28.5 lanes an instruction), 740 us at N = 1e6, p = 4.
+// 207 -> 161 us at N = 1e5, p = 6 (captured with cold caches 173 us: 60 % of the
+// issue slots and 58 % of the FP32 pipe busy, 28.6 lanes an instruction, four
+// blocks per SM), 740 us at N = 1e6, p = 4.
 //
 // Every lane adds its FP32 partial sums (two running sums, one per half of
 // the packed registers, of at most 32 terms each) to double-float totals
@@ -274,7 +275,8 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {
         }
         if (since) fold();
         // the groups' totals in group order
-        const float f0[6] = {h0[0], h0[1], h0[2], l0[0], l0[1], l0[2]}, f1[6] = {h1[0], h1[1], h1[2], l1[0], l1[1], l1[2]};
+        const float f0[6] = {h0[0], h0[1], h0[2], l0[0], l0[1], l0[2]};
+        const float f1[6] = {h1[0], h1[1], h1[2], l1[0], l1[1], l1[2]};
         for (int q = 1; q < G; q++) {
             const int from = min(31, q * L + lane);   // (lanes past the first group add values of no use)
 #pragma unroll
@@ -309,14 +311,21 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {
 // takes 32 as two pulls.  Of an item's entries those with a later leaf count
 // (and the leaf itself, one way).  A block takes an item, each warp a quarter
 // of its targets (a pair of leaves keeps one warp's share of the pipe busy for
-// half a millisecond) and all its sources, 32 at a time, one per lane, so that all
-// lanes work whatever the leaves' sizes.  A warp goes through its m targets with
-// lane l starting at target l mod m: the lanes' pulls on the targets go to distinct places of the warp's
-// sums in shared memory (lanes that would meet have copies of the sums), those on the lane's source stay in registers.  Both are added to the
-// moonlets' sums in memory with FP64 atomics.  N = 1e5, p = 6, beside M2L:
-// 3.57 ms one way (a block per leaf and share, 97 % of the lanes at work), 2.6 ms
-// this way; both near their instructions' time.  With a warp's items cut by
-// entries instead (few sources, many targets) 3.2 ms, and at N = 1e4 twice the one-way time.
+// half a millisecond) and all its sources, 32 at a time, one per lane, so that
+// all lanes work whatever the leaves' sizes.  A warp goes through its m targets
+// with lane l starting at target l mod m: the lanes' pulls on the targets go to
+// distinct places of the warp's sums in shared memory (lanes that would meet
+// have copies of the sums), those on the lane's source stay in registers.  Both
+// are added to the moonlets' sums in memory with FP64 atomics, so a sum's last
+// bits depend on the order of the blocks and of the targets (the far kernel
+// gives coincident moonlets one result).  With few targets to a leaf some of
+// the block's warps have none, and yet no force call of leaves of 1 to 16
+// moonlets takes longer than with a block of 128 threads per leaf (N = 1e5,
+// leaves of one: 8.4 -> 6.3 ms).
+// N = 1e5, p = 6, beside M2L: 3.57 ms one way (a block per leaf and share, 97 %
+// of the lanes at work), 2.6 ms this way; both near their instructions' time.
+// With a warp's items cut by entries instead (few sources, many targets)
+// 3.2 ms, and at N = 1e4 twice the one-way time.
 constexpr int NEAR64_SHARE = 64 / NEAR_WARPS, NEAR64_SUMS = 3 * NEAR64_SHARE;   // targets and sums of a warp
 
 struct __align__(16) NearShared64 {             // of a warp
@@ -357,7 +366,8 @@ __global__ void __launch_bounds__(NEAR_THREADS, 6) k_near_f64(NearArgs A) {
             if (at + lane < I.s1) e = __ldg(&A.p2p_src[at + lane]);
             const bool own = e.x <= I.first && I.first < e.x + e.y;
             const unsigned which = __ballot_sync(0xffffffffu, own);
-            const int o0 = __shfl_sync(0xffffffffu, e.x, __ffs(which) - 1), o1 = o0 + __shfl_sync(0xffffffffu, e.y, __ffs(which) - 1);
+            const int o0 = __shfl_sync(0xffffffffu, e.x, __ffs(which) - 1);
+            const int o1 = o0 + __shfl_sync(0xffffffffu, e.y, __ffs(which) - 1);
             const unsigned keep = __ballot_sync(0xffffffffu, e.y > 0 && (own || e.x > I.first));
             const unsigned from = __fns(keep, 0, lane + 1);   // (a window's entries are not empty)
             e.x = __shfl_sync(0xffffffffu, e.x, from & 31);

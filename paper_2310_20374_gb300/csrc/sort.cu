@@ -768,7 +768,9 @@ static SampleArgs sample_args(const RadixArgs &radix, SampleScratch *scr, long l
 }
 
 // The grid of a sample sort: a block per bucket or per 512 keys, to the cooperative limit.
-static int sample_grid(int n, int most) { return std::max(1, std::min(most, std::max(sample_buckets(n), (n + 511) / 512))); }
+static int sample_grid(int n, int most) {
+    return std::max(1, std::min(most, std::max(sample_buckets(n), (n + 511) / 512)));
+}
 
 // The epoch at which a context's sorts clear their status words: the constant
 // above, or a smaller value from NCORP_RADIX_EPOCH_LIMIT (read at context
@@ -783,9 +785,10 @@ unsigned radix_epoch_limit() {
 }
 
 // Layout of the context's radix scratch (ints): two sets of digit histograms
-// of every pass at [0, 2 RS_MAX_PASSES 256), the epoch counter at RS_EPOCH_AT, the sample
-// sort's buckets at RS_SAMPLE_AT, the tile status words from RS_STATUS_AT on.  The status words never share memory with anything
-// else, so a word left by an earlier sort (of any size) carries an older tag.
+// of every pass at [0, 2 RS_MAX_PASSES 256), the epoch counter at RS_EPOCH_AT,
+// the sample sort's buckets at RS_SAMPLE_AT, the tile status words from
+// RS_STATUS_AT on.  The status words never share memory with anything else, so
+// a word left by an earlier sort (of any size) carries an older tag.
 constexpr int RS_EPOCH_AT = 2 * RS_MAX_PASSES * 256;
 constexpr int RS_SAMPLE_AT = RS_EPOCH_AT + 64;
 constexpr int RS_STATUS_AT = RS_SAMPLE_AT + static_cast<int>(sizeof(SampleScratch) / sizeof(int));

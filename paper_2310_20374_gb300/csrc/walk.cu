@@ -181,7 +181,8 @@ __device__ void walk_lists(const WalkArgs &A, int *s_tmp, unsigned &bar) {
             // the near field's items: a subset of the leaf's moonlets and an equal share of its entries each
             const int m = vp > 0 ? __ldg(&A.count[i]) : 0;
             int parts = 0;
-            for (int t = 0; t < m; t += near_targets(m - t, A.fp64)) parts += near_shares(vp, near_targets(m - t, A.fp64), n_leaves, A.fp64);
+            for (int t = 0; t < m; t += near_targets(m - t, A.fp64))
+                parts += near_shares(vp, near_targets(m - t, A.fp64), n_leaves, A.fp64);
             int total_items = 0;
             const int xi = block_prefix(parts, s_tmp, &total_items);
             if (threadIdx.x == 0) s_items = total_items ? atomicAdd(&A.ctl->n_near, total_items) : 0;
@@ -750,13 +751,15 @@ void launch_walk(ncorp_ctx *c, bool gravity, bool collisions, const int *gate) {
     int per_sm = 0;
     NCORP_CUDA_CHECK(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, WALK_THREADS, 0));
     if (per_sm < 1) per_sm = 1;
-    // (four blocks per SM take 300 us instead of 375 alone at N = 1e6, but in a step the launch waits for room
-    // beside the multipoles: the step 2610 -> 2910 us)
+    // (four blocks per SM take 300 us instead of 375 alone at N = 1e6, but in a
+    // step the launch waits for room beside the multipoles: the step 2610 -> 2910 us)
     if (per_sm > 2) per_sm = 2;
-    // A block per 160 moonlets up to one per SM, then one per 640 up to the cooperative limit; at least 32.  Frontiers
-    // peak near a third of n pairs, several n with the smaller thresholds of low orders: the step with impacts at
-    // N = 3e4, p = 3 takes 591 us at 46 blocks and 505 at 188, the one at 5e4 405 (78) and 392 (304); with 304 blocks
-    // at N = 1e5 the launch waits for room beside the multipoles (541 us at 156, 556 at 304).
+    // A block per 160 moonlets up to one per SM, then one per 640 up to the
+    // cooperative limit; at least 32.  Frontiers peak near a third of n pairs,
+    // several n with the smaller thresholds of low orders: the step with impacts
+    // at N = 3e4, p = 3 takes 591 us at 46 blocks and 505 at 188, the one at 5e4
+    // 405 (78) and 392 (304); with 304 blocks at N = 1e5 the launch waits for
+    // room beside the multipoles (541 us at 156, 556 at 304).
     const int n = c->cur_n;
     const int grid = std::min(coop_blocks(c, per_sm), std::max({32, std::min(n / 160, c->num_sms), n / 640}));
     if (gravity && collisions) k_walk_head<true, true><<<1, HEAD_THREADS, 0, c->stream>>>(A);
