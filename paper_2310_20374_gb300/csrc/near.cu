@@ -218,10 +218,11 @@ __global__ void __launch_bounds__(NEAR_THREADS, 4) k_near_f32(NearArgs A) {
 #pragma unroll
             for (int r = 0; r < 2; r++) {
                 const int j = W.moonlet(pos + 32 * r, lane);
-                // (a place past the window, which a last chunk's padding to quads sums: a massless source at one of
-                // the item's own moonlets, so that its separations are as finite as the leaf's)
-                ph[r] = j >= 0 ? A.hi4[j] : make_float4(th0.x, th0.y, th0.z, 0.f);
-                pl[r] = j >= 0 ? A.lo4[j] : tl0;
+                // (a place past the window, which a last chunk's padding to quads sums: a massless source at the
+                // item's first moonlet, so that its separations are as finite as the leaf's)
+                ph[r] = A.hi4[j >= 0 ? j : I.first];
+                pl[r] = A.lo4[j >= 0 ? j : I.first];
+                if (j < 0) ph[r].w = 0.f;
             }
         };
         if (at < I.s1) {
