@@ -238,9 +238,11 @@ void ensure_tree_capacity(ncorp_ctx *c, int n) {
     const int self = std::max(cc, c->floor_self);
     // Near-field items: an estimate.  A leaf's entries count once per subset of its moonlets (two subsets of 33 to
     // 52 moonlets, one per 64 of more; FP64: one per 16 of up to 256) and are cut into shares of 4 (FP64: 12)
-    // entries or more, the smallest in the smallest trees.  Leaves of more than 64 moonlets at a small theta can
-    // need more, up to several items an entry: they then grow this list alone (n_near tells how many).
-    const int near = std::max(p2p / 2 + 2 * self, c->floor_near);
+    // entries or more, the smallest in the smallest trees.  Leaves of more than 64 moonlets at a small theta can need
+    // more, up to several items an entry: their first call grows this list alone (n_near tells how many) and runs
+    // once more.  (Twice this room spares leaves of 128 to 512 at theta = 0.2 that, and costs every first step whose
+    // lists are allocated anew 0.05 to 0.1 ms: N = 3e4, p = 3 2.50 -> 2.56 ms.)
+    const int near = std::max(p2p / 4 + 2 * self, c->floor_near);
     if (c->wl.front_cap < front || c->wl.m2l_cap < m2l || c->wl.p2p_cap < p2p || c->wl.self_cap < self ||
         c->wl.near_cap < near)
         alloc_lists(c, std::max(front, c->wl.front_cap), std::max(m2l, c->wl.m2l_cap), std::max(p2p, c->wl.p2p_cap),
