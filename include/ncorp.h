@@ -24,6 +24,13 @@
  *     synchronises that stream before it returns (to read the status word),
  *     so outputs are ready when the call returns.
  *   - Units are the caller's; the configuration fixes G and the central mass.
+ *   - Repeatability: keys, orders, trees, geometry, walk decisions, colliding
+ *     pairs and resolved impacts are the same in every run.  Accelerations are
+ *     sums whose order follows atomics (the order of a cell's lists in both
+ *     precisions; the addition of near-field sums in every FP64 evaluation and
+ *     for leaves whose direct list is split in a mixed one), so two runs on the
+ *     same input agree to rounding, not to the last bit.  Coincident moonlets
+ *     of one disk always get one acceleration, bit for bit.
  *   - Invalid arguments (n < 1, p outside 1..6, theta outside (0,1), dt <= 0
  *     where a time step is needed, null pointers, non-finite inputs) return
  *     NCORP_EINVAL before any device work.
@@ -49,7 +56,11 @@ extern "C" {
 #define NCORP_FP64  0        /* every stage in FP64 */
 #define NCORP_MIXED 1        /* multipoles, M2L, P2P, L2L/L2P in FP32 with per-cell scaling;
                                 positions, velocities, kicks/drifts, external forces, keys,
-                                tree geometry and the collision test in FP64 */
+                                tree geometry and the collision test in FP64.  The near field is
+                                not rescaled: choose units in which moonlets that do not coincide
+                                are 1e-10 to 1e12 from their neighbours (closer pairs pull as if
+                                softened), G m is below 1e8 and G m / d^3 of neighbours above
+                                1e-37 (FP32 products: beyond, terms are lost or overflow) */
 
 typedef struct ncorp_ctx ncorp_ctx;
 
@@ -269,8 +280,9 @@ int ncorp_get_state(ncorp_ctx *ctx, double *positions, double *velocities);
 #define NCORP_STAT_GRAPH       16   /* 1 if the last ncorp_step ran as a replayed (or just captured) CUDA graph */
 #define NCORP_STAT_SORT_PATH   17   /* key sort of the last tree: 1 nearly-sorted merge (steps) with the
                                        out-of-place keys ranked (at most 4096 of them), 2 the same with
-                                       them radix-sorted (at most 65536), 0 radix sort of all keys, -1 radix
-                                       sort after the merge found the kept keys out of order */
+                                       them radix-sorted (at most 65536), 0 sort of all keys (sample or
+                                       radix sort), -1 radix sort after the merge found the kept keys out
+                                       of order */
 #define NCORP_STAT_RESOLVED    18   /* impacts resolved by the last ncorp_step (resolve_f > 0) */
 #define NCORP_STAT_FUSED       19   /* 1 if the last ncorp_step's collision search tested the pairs listed by
                                        the previous step's fused walk (fused_walk = 1, no bound exceeded) */
@@ -284,7 +296,7 @@ int ncorp_stats(ncorp_ctx *ctx, int64_t *stats, int n_stats);
  * context's stream around its stages and ncorp_stage_times() returns the
  * device milliseconds each stage took in the last call (summed when a stage
  * runs more than once).  Off by default; on costs a few event records. */
-#define NCORP_STAGE_SORT     0   /* bounding box, keys, radix sort, gather */
+#define NCORP_STAGE_SORT     0   /* bounding box, keys, their sort, gather */
 #define NCORP_STAGE_BUILD    1   /* octree build, leaf list */
 #define NCORP_STAGE_CLIMB    2   /* gravity climb: geometry, theta(M), r_crit; multipoles beside them */
 #define NCORP_STAGE_WALK     3   /* gravity walk and per-target lists */
@@ -455,7 +467,7 @@ int ncorp_fma_peak(int device, int precision, void *cuda_stream, double *flop_pe
 /* Hilbert keys of n moonlets and their stable sort, without allocating any
  * memory: the key and sort stages of a step (the root cube around the
  * bounding box, 21-bit quantisation per axis and a 63-bit 3-D Hilbert key,
- * then the stable radix sort by (key, index)).  The paper has no
+ * then the stable sort by (key, index)).  The paper has no
  * counterpart: this entry point exists for
  * callers that must not allocate device memory once they are set up (a fixed
  * device-memory budget, or a loop in which the implicit synchronisation of
@@ -470,7 +482,7 @@ int ncorp_fma_peak(int device, int precision, void *cuda_stream, double *flop_pe
  * Results are bit-identical to the keys and order that ncorp_tree_export
  * reports after ncorp_accel on the same positions.
  * Scratch: one file-scope device array per device, sized for
- * NCORP_STATIC_MAX_N moonlets (about 3.4 MB); nothing is allocated or freed.
+ * NCORP_STATIC_MAX_N moonlets (about 3.5 MB); nothing is allocated or freed.
  * The call synchronises its stream to read the status word, so it cannot be
  * part of a CUDA graph capture.  The first call on a device looks up the
  * array's address (cudaGetSymbolAddress) with that device current.

@@ -107,8 +107,8 @@ __device__ __forceinline__ void near_store(const NearArgs &A, int i, bool whole,
 // operations per issue slot, the same rounding as the scalar ones): 15 issue
 // slots a pair, below the pipe's 21 cycles.  The next chunk's positions are
 // loaded into registers before the current chunk is summed.  Measured alone:
-// 207 -> 161 us at N = 1e5, p = 6 (captured with cold caches 173 us: 60 % of the
-// issue slots and 58 % of the FP32 pipe busy, 28.6 lanes an instruction, four
+// 207 -> 161 us at N = 1e5, p = 6 (as captured, caches cold: 163 us, 60 % of the
+// issue slots and 59 % of the FP32 pipe busy, 28.5 lanes an instruction, four
 // blocks per SM), 740 us at N = 1e6, p = 4.
 //
 // Every lane adds its FP32 partial sums (two running sums, one per half of
